@@ -78,7 +78,7 @@ struct Dev {
     unsigned *bstart;      // total blocks: first sorted slot of each occupied block
     unsigned *occ;         // occupied blocks being collected by the binning kernel
     unsigned *plan;        // occupied blocks of the grouping in use
-    int4 *chunks;          // work items the substep kernel reads: (block key, first index, count, list)
+    int4 *chunks;          // work items the substep kernel reads: (block key, first index, count, item_word)
     unsigned *ctr;         // device counters, see CTR_*
     int chunk_ctr;         // index in ctr of the number of work items (CTR_N_CHUNKS unless direct)
     // list 0 of a work item: `sorted` (the counting sort, or a direct binning's
@@ -137,6 +137,24 @@ __device__ __forceinline__ void key_coords(const Dev &D, unsigned key, int &inst
     bx = r / D.NB[1];
 }
 
+// Last word of a work item: the coordinates of its block (10 bits each; a
+// grid has at most 1024 blocks per axis) and, in the sign bit, which list the
+// item reads.  The kernels that walk the items read the coordinates instead
+// of dividing the key, three integer divisions per thread and item.
+__device__ __forceinline__ int item_word(int bx, int by, int bz, int list) {
+    return bx | (by << 10) | (bz << 20) | (list << 31);
+}
+__device__ __forceinline__ void item_coords(int w, int &bx, int &by, int &bz) {
+    bx = w & 1023;
+    by = (w >> 10) & 1023;
+    bz = (w >> 20) & 1023;
+}
+__device__ __forceinline__ int item_list(int w) { return w < 0 ? 1 : 0; }
+// key of the block at offset (dx, dy, dz) blocks from the block of `key`, in the same instance
+__device__ __forceinline__ unsigned key_offset(const Dev &D, unsigned key, int dx, int dy, int dz) {
+    return key + (unsigned)((dx * D.NB[1] + dy) * D.NB[2] + dz);
+}
+
 // base cell of a position along one axis; identical arithmetic everywhere a
 // particle is binned or transferred
 __device__ __forceinline__ int base_cell(float x, float inv_dx, float &fx) {
@@ -161,7 +179,7 @@ __device__ __forceinline__ int base_cell_q(int q, const Dev &D, float &fx) {
 __device__ __forceinline__ int advance_q(int q, float v, const Dev &D) {
     float dq = D.dt * v * D.inv_dx * D.q_cell;
     dq = fminf(fmaxf(dq, -1.0e9f), 1.0e9f);          // NaN becomes a bound too
-    const long long s = (long long)q + (long long)__float2ll_rn(dq);
+    const long long s = (long long)q + __float2int_rn(dq);
     return (int)(s < -2147483647ll ? -2147483647ll : (s > 2147483647ll ? 2147483647ll : s));
 }
 

@@ -14,6 +14,8 @@
 // the block's pool slot), and k_between (grid update, chunks from the list
 // counts, activation of the next buffer) replaces plan and sort:
 //   ... -> [k_between(s) -> G2P(s) fused with P2G(s+1) + list write] -> ...
+#include <cstddef>
+
 #include "mpm_dev.cuh"
 #include "mpm_internal.h"
 #include "mpm_math.cuh"
@@ -85,9 +87,9 @@ __global__ void k_load(Dev D, const float *__restrict__ x, const float *__restri
 // binning helpers
 // ---------------------------------------------------------------------------
 
-// Particle block key from its fixed-point position; false when the stencil
-// leaves the grid.
-__device__ __forceinline__ bool particle_key(const Dev &D, int q0, int q1, int q2, int inst, unsigned &key) {
+// Particle block coordinates from its fixed-point position; false when the
+// stencil leaves the grid.
+__device__ __forceinline__ bool particle_block(const Dev &D, int q0, int q1, int q2, int &c0, int &c1, int &c2) {
     float f;
     int b0 = base_cell_q(q0, D, f), b1 = base_cell_q(q1, D, f), b2 = base_cell_q(q2, D, f);
     bool ok = b0 >= 0 && b1 >= 0 && b2 >= 0 && b0 <= D.R[0] - 3 && b1 <= D.R[1] - 3 && b2 <= D.R[2] - 3;
@@ -96,7 +98,9 @@ __device__ __forceinline__ bool particle_key(const Dev &D, int q0, int q1, int q
         b1 = min(max(b1, 0), D.R[1] - 3);
         b2 = min(max(b2, 0), D.R[2] - 3);
     }
-    key = block_key(D, inst, b0 >> 2, b1 >> 2, b2 >> 2);
+    c0 = b0 >> 2;
+    c1 = b1 >> 2;
+    c2 = b2 >> 2;
     return ok;
 }
 
@@ -107,6 +111,8 @@ __device__ __forceinline__ bool particle_key(const Dev &D, int q0, int q1, int q
 struct BinTicket {
     unsigned peers, base, key;
 };
+// mask of a warp's first n lanes
+__device__ __forceinline__ unsigned lanes_below(int n) { return n >= 32 ? 0xffffffffu : (1u << n) - 1u; }
 __device__ __forceinline__ BinTicket bin_begin(const Dev &D, unsigned mask, unsigned key) {
     BinTicket t;
     t.key = key;
@@ -115,19 +121,25 @@ __device__ __forceinline__ BinTicket bin_begin(const Dev &D, unsigned mask, unsi
     if ((int)(threadIdx.x & 31) == __ffs(t.peers) - 1) t.base = atomicAdd(&D.bcount[key], (unsigned)__popc(t.peers));
     return t;
 }
-__device__ __forceinline__ void bin_end(const Dev &D, const BinTicket &t, unsigned p) {
-    const int leader = __ffs(t.peers) - 1;
-    if ((int)(threadIdx.x & 31) == leader && t.base == 0) {
-        unsigned slot = atomicAdd(&D.ctr[CTR_N_OCC], 1u);
-        D.occ[slot] = t.key;
-    }
-    const unsigned base = __shfl_sync(t.peers, t.base, leader);
+// The first particle of a block claims an entry of the occupied list and,
+// apart from it so that the claim's latency can be hidden too, writes it.
+constexpr unsigned NO_ENTRY = 0xffffffffu;
+__device__ __forceinline__ bool first_of_block(const BinTicket &t) {
+    return (int)(threadIdx.x & 31) == __ffs(t.peers) - 1 && t.base == 0;
+}
+__device__ __forceinline__ unsigned bin_rank(const BinTicket &t) {
+    return __shfl_sync(t.peers, t.base, __ffs(t.peers) - 1) + __popc(t.peers & lanemask_lt());
+}
+__device__ __forceinline__ unsigned bin_end(const Dev &D, const BinTicket &t, unsigned p) {
+    const unsigned entry = first_of_block(t) ? atomicAdd(&D.ctr[CTR_N_OCC], 1u) : NO_ENTRY;
     D.key[p] = t.key;
-    D.rank[p] = base + __popc(t.peers & lanemask_lt());
+    D.rank[p] = bin_rank(t);
+    return entry;
 }
 __device__ __forceinline__ void bin_particle(const Dev &D, unsigned mask, unsigned p, unsigned key) {
     BinTicket t = bin_begin(D, mask, key);
-    bin_end(D, t, p);
+    const unsigned entry = bin_end(D, t, p);
+    if (entry != NO_ENTRY) D.occ[entry] = key;
     // the largest block count (sizes the per-block lists of the direct binning)
     if ((int)(threadIdx.x & 31) == __ffs(t.peers) - 1) atomicMax(&D.ctr[CTR_MAX_COUNT], t.base + __popc(t.peers));
 }
@@ -136,13 +148,9 @@ __device__ __forceinline__ void bin_particle(const Dev &D, unsigned mask, unsign
 // a block with pool slot sl goes to slist[par][sl * slist_cap + r]; one whose
 // list is full (r >= slist_cap) or whose slot lies beyond the lists (or is not
 // active, a broken grouping already reported) goes to an overflow entry.
-__device__ __forceinline__ void bin_end_direct(const Dev &D, const BinTicket &t, unsigned p, int slot, int par) {
-    const int leader = __ffs(t.peers) - 1;
-    if ((int)(threadIdx.x & 31) == leader && t.base == 0) {
-        const unsigned i = atomicAdd(&D.ctr[CTR_D_OCC + par], 1u);
-        D.occd[par][i] = t.key;
-    }
-    const unsigned rank = __shfl_sync(t.peers, t.base, leader) + __popc(t.peers & lanemask_lt());
+__device__ __forceinline__ unsigned bin_end_direct(const Dev &D, const BinTicket &t, unsigned p, int slot, int par) {
+    const unsigned entry = first_of_block(t) ? atomicAdd(&D.ctr[CTR_D_OCC + par], 1u) : NO_ENTRY;
+    const unsigned rank = bin_rank(t);
     if (slot >= 0 && (unsigned)slot < D.slist_blocks && rank < D.slist_cap) {
         D.slist[par][(size_t)slot * D.slist_cap + rank] = p;
     } else {
@@ -155,6 +163,7 @@ __device__ __forceinline__ void bin_end_direct(const Dev &D, const BinTicket &t,
             set_err(D, ERRB_CAPACITY);
         }
     }
+    return entry;
 }
 
 __global__ void k_bin(Dev D) {
@@ -166,9 +175,9 @@ __global__ void k_bin(Dev D) {
         if (!valid) continue;
         float4 r0 = D.rec[(size_t)p * REC_F4];
         int inst = __float_as_int(D.rec[(size_t)p * REC_F4 + 7].z);
-        unsigned key;
-        if (!particle_key(D, rec_q(r0.x), rec_q(r0.y), rec_q(r0.z), inst, key)) set_err(D, ERRB_DOMAIN);
-        bin_particle(D, mask, (unsigned)p, key);
+        int c0, c1, c2;
+        if (!particle_block(D, rec_q(r0.x), rec_q(r0.y), rec_q(r0.z), c0, c1, c2)) set_err(D, ERRB_DOMAIN);
+        bin_particle(D, mask, (unsigned)p, block_key(D, inst, c0, c1, c2));
     }
 }
 
@@ -227,9 +236,12 @@ __global__ void __launch_bounds__(1024) k_plan(Dev D, int bump_mask) {
             D.bstart[key] = start;
             D.plan[i] = key;
             D.bcount[key] = 0;
+            int inst, bx, by, bz;
+            key_coords(D, key, inst, bx, by, bz);
+            const int w = item_word(bx, by, bz, 0);
             for (unsigned j = 0; j < nch; ++j) {
                 unsigned ci = tchunks + ek + j;
-                if (ci < D.max_chunks) D.chunks[ci] = make_int4((int)key, (int)(start + j * CH), (int)min(CH, cnt - j * CH), 0);
+                if (ci < D.max_chunks) D.chunks[ci] = make_int4((int)key, (int)(start + j * CH), (int)min(CH, cnt - j * CH), w);
                 else set_err(D, ERRB_CAPACITY);
             }
         }
@@ -415,10 +427,13 @@ __global__ void k_between(Dev D, int upd, int act) {
             }
             const unsigned nch = (main + CH - 1) / CH;
             const unsigned c0 = warp_claim(&D.ctr[CTR_D_CH + upd], nch);
+            int inst, bx, by, bz;
+            key_coords(D, key, inst, bx, by, bz);
+            const int w = item_word(bx, by, bz, 0);
             for (unsigned j = 0; j < nch; ++j) {
                 if (c0 + j < D.max_chunks_d)
                     D.chunksd[upd][c0 + j] = make_int4((int)key, (int)((unsigned)sl * D.slist_cap + j * CH),
-                                                       (int)min(CH, main - j * CH), 0);
+                                                       (int)min(CH, main - j * CH), w);
                 else
                     set_err(D, ERRB_CAPACITY);
             }
@@ -426,8 +441,14 @@ __global__ void k_between(Dev D, int upd, int act) {
             const unsigned o = w0 - e1 + lane;
             const unsigned c = warp_claim(&D.ctr[CTR_D_CH + upd], o < novf ? 1u : 0u);
             if (o >= novf) continue;
-            if (c < D.max_chunks_d) D.chunksd[upd][c] = make_int4((int)D.ovf[upd][2 * o + 1], (int)(2 * o), 1, 1);
-            else set_err(D, ERRB_CAPACITY);
+            if (c < D.max_chunks_d) {
+                const unsigned key = D.ovf[upd][2 * (size_t)o + 1];
+                int inst, bx, by, bz;
+                key_coords(D, key, inst, bx, by, bz);
+                D.chunksd[upd][c] = make_int4((int)key, (int)(2 * o), 1, item_word(bx, by, bz, 1));
+            } else {
+                set_err(D, ERRB_CAPACITY);
+            }
         } else {   // activation of act: one neighbour of an occupied block
             activate_item(D, D.occd[upd], w0 - e2 + lane, nocc * 27u, act, ep_new);
         }
@@ -461,8 +482,17 @@ __global__ void k_between(Dev D, int upd, int act) {
 //      the fixed-point tile the warps take the packets ordered by (rank
 //      within bank, bank of the base node): one loop iteration moves every
 //      lane by the same node offset, so lanes with distinct base banks hit
-//      distinct banks in all 108 atomics, and the first warps of a chunk see
-//      at most two-way conflicts.
+//      distinct banks in all 108 atomics.  The particles are binned in that
+//      order too, so a list keeps it: the direct-binning substeps that follow
+//      (OWN) scatter each thread's own particle from registers in list order,
+//      without packets, their sort and two of the five barriers, and their
+//      gather reads distinct banks as well.
+// What bounds it: the shared-memory data pipe (70% busy at 300k particles
+// before the gather tile became planes, the tile strides covered all banks and
+// the unread v and C stores went; 59% after) and, with 16 warps per SM, the
+// latency of one particle's dependent chain.  Fused launch 62.5 -> 53.4 us at
+// 300k particles on 128^3 and 356 -> 297 us at 2M on 256^3 (53 and 58% of the
+// issue slots unused; DRAM 8 and 21%).
 // SCAT selects the scatter of phase B: 0 = float shared-memory atomics;
 // 1 = int32 fixed-point shared-memory atomics with a per-chunk scale (native
 // integer atomics; the scale keeps the rounding below 2^-30 of the chunk's
@@ -474,14 +504,29 @@ constexpr int GT = 6;    // gather tile edge (nodes 4B .. 4B+5)
 constexpr int GT3 = GT * GT * GT;
 constexpr int ST = 8;    // scatter tile edge (nodes 4B-1 .. 4B+6)
 constexpr int ST3 = ST * ST * ST;
-constexpr int STP = ST + 1;            // padded row of the fixed-point tile (breaks bank aliasing)
-constexpr int ST3P = ST * ST * STP;
+// Strides of the fixed-point tile, in words: 1 along k, 8 along j, 68 along i.
+// The 64 base cells of a block then cover the 32 banks exactly twice each
+// (j fills banks 0-3, 8-11, 16-19, 24-27; an odd i shifts by 4), where the
+// former strides 9 and 72 left four banks unused and put up to four cells in one.
+constexpr int STI = ST * ST + 4;
+constexpr int ST3P = ST * STI;         // 544 = 17 x 32: every component starts at bank 0
 constexpr int CH_MAX = 128;            // particles per chunk (one per thread)
-__device__ __forceinline__ int tidx(int i, int j, int k) { return (i * ST + j) * STP + k; }
+__device__ __forceinline__ int tidx(int i, int j, int k) { return i * STI + j * ST + k; }
 
-__device__ __forceinline__ int page_slot(const Dev &D, int par, unsigned ep, int inst, int bx, int by, int bz) {
-    if (bx < 0 || by < 0 || bz < 0 || bx >= D.NB[0] || by >= D.NB[1] || bz >= D.NB[2]) return -1;
-    unsigned k = block_key(D, inst, bx, by, bz);
+// Strides of the gather tile, in nodes: 1, 8, 52.  As in the fixed-point tile
+// the 64 base cells cover the banks evenly, and lanes whose scatter banks
+// differ (the order a particle list has, see phase B) differ here too.
+constexpr int GTI = GT * ST + 4;
+constexpr int GTP3 = GT * GTI;
+__device__ __forceinline__ int gtidx(int i, int j, int k) { return i * GTI + j * ST + k; }
+
+// pool slot of the block at (bx + dx, by + dy, bz + dz), key: that of (bx, by, bz)
+__device__ __forceinline__ int page_slot(const Dev &D, int par, unsigned ep, unsigned key, int bx, int by, int bz,
+                                         int dx, int dy, int dz) {
+    if ((unsigned)(bx + dx) >= (unsigned)D.NB[0] || (unsigned)(by + dy) >= (unsigned)D.NB[1] ||
+        (unsigned)(bz + dz) >= (unsigned)D.NB[2])
+        return -1;
+    const unsigned k = key_offset(D, key, dx, dy, dz);
     // both words are loaded before either is tested: one round trip
     const unsigned e = D.page_epoch[par][k];
     const int sl = D.page[par][k];
@@ -494,8 +539,8 @@ constexpr int PK_F4 = 5;          // scatter packet: X(3) m | P(3) - | Ad(9) (+3
 constexpr int RS_F4 = REC_F4 + 1; // staged record stride: 144 B keeps per-thread float4 reads conflict-free
 template <int TPB> struct SubstepSmem {
     float4 rec[TPB * RS_F4];         // the chunk's records, staged ahead of use
-    float4 pk[TPB * PK_F4];          // scatter packets of the chunk's particles
-    float4 g[GT3];                   // gather tile: (v, m) per node
+    float2 gxy[GTP3];                // gather tile: v0, v1 per node
+    float gz[GTP3];                  // ... and v2
     union {
         float f[4 * ST3P];           // scatter tile, component-major [m0 | m1 | m2 | m], padded rows
         int i[4 * ST3P];
@@ -506,17 +551,24 @@ template <int TPB> struct SubstepSmem {
     int ps[35];                      // ... and pool slot; 0..26 scatter blocks, 27..34 gather blocks
     int slot_s[2][27];               // pool slot of blocks (B-1 .. B+1)^3 in the scatter grid, per chunk parity
     float red[2 * (TPB / 32)];
-    float scale[2];
+    // the rest is not used (nor allocated) where each thread scatters its own particle
     int ccount[32];                  // packets per bank of their base node (scatter order)
+    float4 pk[TPB * PK_F4];          // scatter packets of the chunk's particles
     int ptab[TPB];                   // packets of rank < r
     unsigned mtab[TPB];              // banks holding a packet of rank r
     int prank[TPB], pcol[TPB];       // each packet's bank and rank within it
     int perm[TPB];                   // scatter order: packets by (rank, bank)
 };
+template <int TPB, bool OWN> constexpr size_t substep_smem() {
+    return OWN ? offsetof(SubstepSmem<TPB>, ccount) : sizeof(SubstepSmem<TPB>);
+}
 
 __device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async8(void *dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(smem_addr(dst)), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async4(void *dst, const void *src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(smem_addr(dst)), "l"(src) : "memory");
@@ -533,9 +585,9 @@ template <int TPB, bool GATHER, bool SCATTER>
 __device__ __forceinline__ void stage_level2(const Dev &D, SubstepSmem<TPB> &S, int4 ch, int gpar, int spar,
                                              unsigned ep_g, unsigned ep_s) {
     const int tid = threadIdx.x;
-    if (tid < ch.z) cp_async4(&S.pidx[tid], (ch.w ? D.ovf_in : D.sorted) + ch.y + tid);
-    int inst, bx, by, bz;
-    key_coords(D, (unsigned)ch.x, inst, bx, by, bz);
+    if (tid < ch.z) cp_async4(&S.pidx[tid], (item_list(ch.w) ? D.ovf_in : D.sorted) + ch.y + tid);
+    int bx, by, bz;
+    item_coords(ch.w, bx, by, bz);
     const int t = tid - (TPB - 64 > 0 ? 64 : 0);    // the lookups go to the last warps of the CTA
     if (t >= 0 && t < 35 && (t < 27 ? SCATTER : GATHER)) {
         int qx, qy, qz, par;
@@ -546,7 +598,7 @@ __device__ __forceinline__ void stage_level2(const Dev &D, SubstepSmem<TPB> &S, 
             S.pe[t] = ep + 1u;
             S.ps[t] = -1;
         } else {
-            const unsigned k = block_key(D, inst, qx, qy, qz);
+            const unsigned k = key_offset(D, (unsigned)ch.x, qx - bx, qy - by, qz - bz);
             cp_async4(&S.pe[t], D.page_epoch[par] + k);
             cp_async4(&S.ps[t], D.page[par] + k);
         }
@@ -568,14 +620,19 @@ __device__ __forceinline__ void stage_level3(const Dev &D, SubstepSmem<TPB> &S, 
         }
     }
     if (GATHER) {
-        int inst, bx, by, bz;
-        key_coords(D, (unsigned)ch.x, inst, bx, by, bz);
         for (int t = tid; t < GT3; t += TPB) {
             const int i = t / (GT * GT), j = (t / GT) % GT, k = t % GT;
             const int b = 27 + (((i >> 2) << 2) | ((j >> 2) << 1) | (k >> 2));
             const int sl = S.pe[b] == ep_g ? S.ps[b] : -1;
-            if (sl >= 0) cp_async16(&S.g[t], D.gv[gpar] + (size_t)sl * BLK_NODES + node_local(i, j, k));
-            else S.g[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+            const int q = gtidx(i, j, k);
+            if (sl >= 0) {
+                const float4 *src = D.gv[gpar] + (size_t)sl * BLK_NODES + node_local(i, j, k);
+                cp_async8(&S.gxy[q], src);
+                cp_async4(&S.gz[q], &src->z);
+            } else {
+                S.gxy[q] = make_float2(0.f, 0.f);
+                S.gz[q] = 0.f;
+            }
         }
     }
 }
@@ -596,12 +653,21 @@ __device__ __forceinline__ void stage_slots(SubstepSmem<TPB> &S, int buf, unsign
 // Sigma plasticity).  Without it the kernel handles fixed-corotated and
 // Neo-Hookean with von Mises / Drucker-Prager only, and its register
 // allocation is not shared with the rarer models.
-template <int MODE, int SCAT, int TPB, bool XM, bool DB>
-__global__ void __launch_bounds__(TPB, 512 / TPB) k_substep(Dev D, int gpar, int spar) {
+// keep: the new v and C go to the particle's record too.  The next gather
+// overwrites both before anything reads them, so a fused substep whose state
+// is not kept (no checkpoint, no tape) leaves them out; a run's last substep
+// writes them.
+// OWN (direct binning, fixed-point scatter): each thread scatters its own
+// particle from registers, in the order of the list, instead of handing
+// packets over in the (rank, bank) order.
+template <int MODE, int SCAT, int TPB, bool XM, bool DB, bool OWN>
+__global__ void __launch_bounds__(TPB, 512 / TPB) k_substep(Dev D, int gpar, int spar, int keep) {
     extern __shared__ float4 smem_raw[];
     SubstepSmem<TPB> &S = *reinterpret_cast<SubstepSmem<TPB> *>(smem_raw);
     constexpr bool GATHER = MODE != MODE_P2G;
     constexpr bool SCATTER = MODE != MODE_G2P;
+    constexpr bool PERM = SCATTER && SCAT == 1 && !OWN;        // packets taken by (rank, bank)
+    constexpr bool ORDERED = GATHER && PERM;                   // particles are binned in that order
     if (DB && blockIdx.x == 0 && threadIdx.x == 0) {
         // counters this kernel does not read and the next launch starts from:
         // the activation count of the gather buffer (activated again next)
@@ -633,7 +699,7 @@ __global__ void __launch_bounds__(TPB, 512 / TPB) k_substep(Dev D, int gpar, int
     }
     if (SCATTER && SCAT != 2)
         for (int t = tid; t < 4 * ST3P; t += T) S.t.i[t] = 0;
-    if (tid < 32) S.ccount[tid] = 0;
+    if (PERM && tid < 32) S.ccount[tid] = 0;
     __syncthreads();
     stage_level2<TPB, GATHER, SCATTER>(D, S, S.cd[0], gpar, spar, ep_g, ep_s);
     cp_async_commit();
@@ -655,13 +721,20 @@ __global__ void __launch_bounds__(TPB, 512 / TPB) k_substep(Dev D, int gpar, int
         if (tid == 0 && cn + gridDim.x < n_chunks) cp_async16(&S.cd[(kc + 2) % 3], D.chunks + cn + gridDim.x);
         if (has_next) stage_level2<TPB, GATHER, SCATTER>(D, S, S.cd[(kc + 1) % 3], gpar, spar, ep_g, ep_s);
         cp_async_commit();
-        int inst, bx, by, bz;
-        key_coords(D, (unsigned)ch.x, inst, bx, by, bz);
+        int bx, by, bz;
+        item_coords(ch.w, bx, by, bz);
         const int ox = bx * BLK, oy = by * BLK, oz = bz * BLK;   // gather tile origin (node)
-        const int rounds = 1;
 
         // ---- A. per-particle update -----------------------------------------
         float bnd_m = 0.f, bnd_v = 0.f;
+        // the scatter packet: tile coordinates of the new position, mass (0:
+        // nothing to scatter), momentum, affine momentum times dx
+        float X0 = 0.f, X1 = 0.f, X2 = 0.f, pm = 0.f, P0 = 0.f, P1 = 0.f, P2 = 0.f;
+        float Ad[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        unsigned entry = NO_ENTRY;
+        BinTicket ticket;
+        unsigned bin_p = 0;
+        int bin_slot = -1;
         {
             const int j = tid;
             const bool valid = j < cnt;
@@ -685,9 +758,8 @@ __global__ void __launch_bounds__(TPB, 512 / TPB) k_substep(Dev D, int gpar, int
                 Cm[8] = r4.x;
             }
             float4 *rp = D.rec + (size_t)p * REC_F4;
-            unsigned key = 0;
             bool in_dom = true;
-            BinTicket ticket;
+            int c0 = 0, c1 = 0, c2 = 0;   // the block of the new position
             if (GATHER) {
                 float f0, f1, f2;
                 int b0 = base_cell_q(q[0], D, f0) - ox, b1 = base_cell_q(q[1], D, f1) - oy,
@@ -714,7 +786,9 @@ __global__ void __launch_bounds__(TPB, 512 / TPB) k_substep(Dev D, int gpar, int
                         float Sij[3] = {0.f, 0.f, 0.f}, Tij[3] = {0.f, 0.f, 0.f};
 #pragma unroll
                         for (int k = 0; k < 3; ++k) {
-                            const float4 g = S.g[((b0 + i) * GT + (b1 + jj)) * GT + (b2 + k)];
+                            const int nd = gtidx(b0 + i, b1 + jj, b2 + k);
+                            const float2 gxy = S.gxy[nd];
+                            const float3 g = make_float3(gxy.x, gxy.y, S.gz[nd]);
                             Sij[0] += w2[k] * g.x; Sij[1] += w2[k] * g.y; Sij[2] += w2[k] * g.z;
                             Tij[0] += wz1[k] * g.x; Tij[1] += wz1[k] * g.y; Tij[2] += wz1[k] * g.z;
                         }
@@ -738,11 +812,15 @@ __global__ void __launch_bounds__(TPB, 512 / TPB) k_substep(Dev D, int gpar, int
 #pragma unroll
                 for (int d = 0; d < 3; ++d) { v[d] = vn[d]; q[d] = advance_q(q[d], vn[d], D); }
                 if (!(isfinite(vn[0]) && isfinite(vn[1]) && isfinite(vn[2]))) set_err(D, ERRB_NONFINITE);
-                in_dom = particle_key(D, q[0], q[1], q[2], inst, key);
-                ticket = bin_begin(D, lane_mask, key);      // result consumed after the SVD
-                rp[1] = make_float4(v[0], v[1], v[2], vol);
-                rp[2] = make_float4(Cm[0], Cm[1], Cm[2], Cm[3]);
-                rp[3] = make_float4(Cm[4], Cm[5], Cm[6], Cm[7]);
+                if (!ORDERED) {   // the atomic's result is consumed after the SVD
+                    in_dom = particle_block(D, q[0], q[1], q[2], c0, c1, c2);
+                    ticket = bin_begin(D, lane_mask, key_offset(D, (unsigned)ch.x, c0 - bx, c1 - by, c2 - bz));
+                }
+                if (MODE == MODE_G2P || keep) {
+                    rp[1] = make_float4(v[0], v[1], v[2], vol);
+                    rp[2] = make_float4(Cm[0], Cm[1], Cm[2], Cm[3]);
+                    rp[3] = make_float4(Cm[4], Cm[5], Cm[6], Cm[7]);
+                }
                 // F <- (I + dt C) F
                 float G[9];
 #pragma unroll
@@ -797,8 +875,20 @@ __global__ void __launch_bounds__(TPB, 512 / TPB) k_substep(Dev D, int gpar, int
                 }
             }
 
-            if (!GATHER) in_dom = particle_key(D, q[0], q[1], q[2], inst, key);
+            if (!GATHER || ORDERED) in_dom = particle_block(D, q[0], q[1], q[2], c0, c1, c2);
             if (!in_dom) set_err(D, ERRB_DOMAIN);
+            // pool slot of the new block in the scatter buffer: one of the
+            // chunk block's 27 neighbours (a particle moves at most a cell);
+            // beyond the neighbourhood (a broken grouping, already reported)
+            // the page table is read, as k_between reads it for the block
+            int slot = -1;
+            if (DB) {
+                const int d0 = c0 - bx + 1, d1 = c1 - by + 1, d2 = c2 - bz + 1;
+                if ((unsigned)d0 < 3u && (unsigned)d1 < 3u && (unsigned)d2 < 3u)
+                    slot = S.slot_s[kc & 1][(d0 * 3 + d1) * 3 + d2];
+                else
+                    slot = page_slot(D, spar, ep_s, (unsigned)ch.x, bx, by, bz, c0 - bx, c1 - by, c2 - bz);
+            }
 
             if (SCATTER) {
                 // Kirchhoff stress of F (App. B.1 / App. A) and the affine momentum
@@ -813,22 +903,21 @@ __global__ void __launch_bounds__(TPB, 512 / TPB) k_substep(Dev D, int gpar, int
                     tau = Sym{0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
                 }
                 const float kf = 4.f * dt * vol * inv_dx * inv_dx;
-                float Ad[9];
                 Ad[0] = (mass * Cm[0] - kf * tau.xx) * dx; Ad[1] = (mass * Cm[1] - kf * tau.xy) * dx;
                 Ad[2] = (mass * Cm[2] - kf * tau.xz) * dx; Ad[3] = (mass * Cm[3] - kf * tau.xy) * dx;
                 Ad[4] = (mass * Cm[4] - kf * tau.yy) * dx; Ad[5] = (mass * Cm[5] - kf * tau.yz) * dx;
                 Ad[6] = (mass * Cm[6] - kf * tau.xz) * dx; Ad[7] = (mass * Cm[7] - kf * tau.yz) * dx;
                 Ad[8] = (mass * Cm[8] - kf * tau.zz) * dx;
-                const float P0 = mass * v[0], P1 = mass * v[1], P2 = mass * v[2];
+                P0 = mass * v[0]; P1 = mass * v[1]; P2 = mass * v[2];
                 // tile-local continuous node coordinate of the new position (the
                 // integer offset is taken off in fixed point; one rounding)
-                const float X0 = (float)(q[0] - ((ox - 1) << D.qf)) * D.q_unit,
-                            X1 = (float)(q[1] - ((oy - 1) << D.qf)) * D.q_unit,
-                            X2 = (float)(q[2] - ((oz - 1) << D.qf)) * D.q_unit;
+                X0 = (float)(q[0] - ((ox - 1) << D.qf)) * D.q_unit;
+                X1 = (float)(q[1] - ((oy - 1) << D.qf)) * D.q_unit;
+                X2 = (float)(q[2] - ((oz - 1) << D.qf)) * D.q_unit;
                 // base cell floor(X - 0.5) in [0, ST-3] keeps the 3^3 stencil in the tile
                 const bool in_tile = in_dom && X0 >= 0.5f && X1 >= 0.5f && X2 >= 0.5f && X0 < (float)ST - 1.5f &&
                                      X1 < (float)ST - 1.5f && X2 < (float)ST - 1.5f;
-                float pm = mass;
+                pm = mass;
                 if (in_dom && !in_tile) {
                     // moved out of the tile: straight to the global grid
                     pm = 0.f;
@@ -845,7 +934,8 @@ __global__ void __launch_bounds__(TPB, 512 / TPB) k_substep(Dev D, int gpar, int
                                 const float d0 = (float)i - f0, d1 = (float)jj - f1, d2 = (float)k - f2;
                                 const float wt = w0[i] * w1[jj] * w2[k];
                                 const int I = g0 + i, J = g1 + jj, K = g2 + k;
-                                const int sl = page_slot(D, spar, ep_s, inst, I >> 2, J >> 2, K >> 2);
+                                const int sl = page_slot(D, spar, ep_s, (unsigned)ch.x, bx, by, bz, (I >> 2) - bx,
+                                                         (J >> 2) - by, (K >> 2) - bz);
                                 if (sl >= 0)
                                     red_add_v4(D.gmv[spar] + (size_t)sl * BLK_NODES + node_local(I, J, K),
                                                wt * (P0 + Ad[0] * d0 + Ad[1] * d1 + Ad[2] * d2),
@@ -865,31 +955,21 @@ __global__ void __launch_bounds__(TPB, 512 / TPB) k_substep(Dev D, int gpar, int
                     const float ap = fmaxf(fabsf(P0), fmaxf(fabsf(P1), fabsf(P2)));
                     bnd_v += pm > 0.f ? ap + 4.5f * am : 0.f;
                 }
+                if (!OWN) {
                 sr[0] = make_float4(X0, X1, X2, pm);
-                sr[1] = make_float4(P0, P1, P2, 0.f);
+                sr[1] = make_float4(P0, P1, P2, __int_as_float(slot));
                 sr[2] = make_float4(Ad[0], Ad[1], Ad[2], Ad[3]);
                 sr[3] = make_float4(Ad[4], Ad[5], Ad[6], Ad[7]);
-                sr[4] = make_float4(Ad[8], 0.f, 0.f, 0.f);
+                sr[4] = make_float4(Ad[8], __uint_as_float(p),
+                                    __uint_as_float(key_offset(D, (unsigned)ch.x, c0 - bx, c1 - by, c2 - bz)), 0.f);
+                }
             }
-            if (DB) {
-                // pool slot of the new block in the scatter buffer: one of the
-                // chunk block's 27 neighbours (a particle moves at most a cell)
-                float fq;
-                const int d0 = (base_cell_q(q[0], D, fq) >> 2) - bx + 1, d1 = (base_cell_q(q[1], D, fq) >> 2) - by + 1,
-                          d2 = (base_cell_q(q[2], D, fq) >> 2) - bz + 1;
-                const bool near = (unsigned)d0 < 3u && (unsigned)d1 < 3u && (unsigned)d2 < 3u;
-                // beyond the neighbourhood (a broken grouping, already reported)
-                // the page table is read, as k_between reads it for the block
-                const int slot = near ? S.slot_s[kc & 1][(d0 * 3 + d1) * 3 + d2]
-                                      : (D.page_epoch[spar][key] == ep_s ? D.page[spar][key] : -1);
-                bin_end_direct(D, ticket, p, slot, spar);
-            } else if (MODE != MODE_P2G) {
-                bin_end(D, ticket, p);
-            }
+            if (!ORDERED && MODE != MODE_P2G)
+                entry = DB ? bin_end_direct(D, ticket, p, slot, spar) : bin_end(D, ticket, p);
             }
         }
 
-        if (SCATTER && SCAT == 1 && tid < cnt) {
+        if (PERM && tid < cnt) {
             // bank of the packet's base node: every node of its stencil is the
             // base plus an offset common to all packets in one loop iteration,
             // and the tile's component stride is a multiple of 32 banks
@@ -913,7 +993,7 @@ __global__ void __launch_bounds__(TPB, 512 / TPB) k_substep(Dev D, int gpar, int
         // gather-tile buffers, so level 3 of chunk c + G goes in flight now
         cp_async_wait_all();
         __syncthreads();
-        if (SCATTER && SCAT == 1) {
+        if (PERM) {
             // per rank level r: the packets of lower rank, and the banks with a packet of rank r
             const int lane = tid & 31, w = tid >> 5;
             const int cc = S.ccount[lane];
@@ -935,48 +1015,62 @@ __global__ void __launch_bounds__(TPB, 512 / TPB) k_substep(Dev D, int gpar, int
         cp_async_commit();
 
         if (SCATTER) {
-            if (SCAT == 1 && tid == 0) {
-                float bm = 0.f, bv = 0.f;
-                for (int w = 0; w < T / 32; ++w) { bm += S.red[w]; bv += S.red[(TPB / 32) + w]; }
-                S.scale[0] = bm > 0.f ? 1073741824.f / bm : 1.f;     // 2^30 / bound
-                S.scale[1] = bv > 0.f ? 1073741824.f / bv : 1.f;
-            }
+            // per-chunk fixed-point scales: 2^30 over the sum of the bounds
+            float sc_m = 1.f, sc_v = 1.f;
             if (SCAT == 1) {
-                __syncthreads();
-                if (tid < cnt) {
-                    const int r = S.prank[tid], k = S.pcol[tid];
-                    S.perm[S.ptab[r] + __popc(S.mtab[r] & ((1u << k) - 1u))] = tid;
-                }
-                if (tid < 32) S.ccount[tid] = 0;
-                __syncthreads();
+                float bm = 0.f, bv = 0.f;
+#pragma unroll
+                for (int w = 0; w < T / 32; ++w) { bm += S.red[w]; bv += S.red[(TPB / 32) + w]; }
+                sc_m = bm > 0.f ? 1073741824.f / bm : 1.f;
+                sc_v = bv > 0.f ? 1073741824.f / bv : 1.f;
             }
-            const float sc_m = SCAT == 1 ? S.scale[0] : 1.f, sc_v = SCAT == 1 ? S.scale[1] : 1.f;
 
             // ---- B. scatter packets -------------------------------------------
-            // lane-transposed mapping: the warp's lanes take packets S/32 apart
-            // (sorted neighbours share a cell and would hit the same nodes)
-            const int span = rounds * (T >> 5);
-            for (int r = 0; r < rounds; ++r) {
-                const int u = r * T + tid;
-                int j;
-                if (SCAT == 1) {
-                    if (u >= cnt) continue;
-                    j = S.perm[u];   // warps take packets by (rank, bank): few bank conflicts
-                } else {
-                    j = (u & 31) * span + (u >> 5);
-                    if (j >= cnt) continue;
+            // (rank, bank) order: few bank conflicts; else lane-transposed: the
+            // warp's lanes take packets T/32 apart (neighbours may share a cell
+            // and hit the same nodes)
+            if (!OWN) {
+                int j = (tid & 31) * (T >> 5) + (tid >> 5);
+                if (PERM) {
+                    __syncthreads();
+                    if (tid < cnt) {
+                        const int r = S.prank[tid], k = S.pcol[tid];
+                        S.perm[S.ptab[r] + __popc(S.mtab[r] & ((1u << k) - 1u))] = tid;
+                    }
+                    if (tid < 32) S.ccount[tid] = 0;
+                    __syncthreads();
+                    j = tid < cnt ? S.perm[tid] : TPB;
                 }
-                const float4 q0 = S.pk[j * PK_F4];
-                if (!(q0.w > 0.f)) continue;
-                const float4 q1r = S.pk[j * PK_F4 + 1], q2 = S.pk[j * PK_F4 + 2], q3 = S.pk[j * PK_F4 + 3],
-                             q4 = S.pk[j * PK_F4 + 4];
+                pm = 0.f;
+                if (j < cnt) {
+                    const float4 q0 = S.pk[j * PK_F4], q1 = S.pk[j * PK_F4 + 1], q2 = S.pk[j * PK_F4 + 2],
+                                 q3 = S.pk[j * PK_F4 + 3], q4 = S.pk[j * PK_F4 + 4];
+                    X0 = q0.x; X1 = q0.y; X2 = q0.z; pm = q0.w;
+                    P0 = q1.x; P1 = q1.y; P2 = q1.z;
+                    Ad[0] = q2.x; Ad[1] = q2.y; Ad[2] = q2.z; Ad[3] = q2.w;
+                    Ad[4] = q3.x; Ad[5] = q3.y; Ad[6] = q3.z; Ad[7] = q3.w;
+                    Ad[8] = q4.x;
+                    // the particle is binned in the scatter's order: its list then
+                    // keeps lanes of a warp in cells of different banks, which the
+                    // next substep's gather and scatter meet in that order.  The
+                    // atomic's result is consumed after the scatter.
+                    if (ORDERED) {
+                        ticket = bin_begin(D, lanes_below(cnt - (tid & ~31)), __float_as_uint(q4.z));
+                        bin_p = __float_as_uint(q4.y);
+                        bin_slot = __float_as_int(q1.w);
+                    }
+                }
+            }
+            if (pm > 0.f) {
                 // the fixed-point scale is folded into the packet (1 for SCAT != 1)
-                const float4 q1 = make_float4(q1r.x * sc_v, q1r.y * sc_v, q1r.z * sc_v, 0.f);
-                const float qm = q0.w * sc_m;
-                const float Ad[9] = {q2.x * sc_v, q2.y * sc_v, q2.z * sc_v, q2.w * sc_v, q3.x * sc_v,
-                                     q3.y * sc_v, q3.z * sc_v, q3.w * sc_v, q4.x * sc_v};
-                const float b0f = floorf(q0.x - 0.5f), b1f = floorf(q0.y - 0.5f), b2f = floorf(q0.z - 0.5f);
-                const float f0 = q0.x - b0f, f1 = q0.y - b1f, f2 = q0.z - b2f;
+                if (SCAT == 1) {
+                    P0 *= sc_v; P1 *= sc_v; P2 *= sc_v;
+#pragma unroll
+                    for (int t = 0; t < 9; ++t) Ad[t] *= sc_v;
+                }
+                const float qm = pm * sc_m;
+                const float b0f = floorf(X0 - 0.5f), b1f = floorf(X1 - 0.5f), b2f = floorf(X2 - 0.5f);
+                const float f0 = X0 - b0f, f1 = X1 - b1f, f2 = X2 - b2f;
                 const int t0 = (int)b0f, t1 = (int)b1f, t2 = (int)b2f;
                 float w0[3], w1[3], w2[3];
                 bspline_w(f0, w0);
@@ -989,8 +1083,8 @@ __global__ void __launch_bounds__(TPB, 512 / TPB) k_substep(Dev D, int gpar, int
                     for (int jj = 0; jj < 3; ++jj) {
                         const float d1 = (float)jj - f1;
                         const float wij = w0[i] * w1[jj];
-                        const float a0 = q1.x + Ad[0] * d0 + Ad[1] * d1, a1 = q1.y + Ad[3] * d0 + Ad[4] * d1,
-                                    a2 = q1.z + Ad[6] * d0 + Ad[7] * d1;
+                        const float a0 = P0 + Ad[0] * d0 + Ad[1] * d1, a1 = P1 + Ad[3] * d0 + Ad[4] * d1,
+                                    a2 = P2 + Ad[6] * d0 + Ad[7] * d1;
 #pragma unroll
                         for (int k = 0; k < 3; ++k) {
                             const float d2 = (float)k - f2;
@@ -1022,12 +1116,20 @@ __global__ void __launch_bounds__(TPB, 512 / TPB) k_substep(Dev D, int gpar, int
                     }
                 }
             }
+            if (ORDERED && tid < cnt)
+                entry = DB ? bin_end_direct(D, ticket, bin_p, bin_slot, spar) : bin_end(D, ticket, bin_p);
             if (SCAT != 2) {
                 __syncthreads();
                 // flush: one vector reduction per node that received mass
                 const float iv = 1.f / sc_v, im = 1.f / sc_m;
-                for (int t = tid; t < ST3; t += T) {
-                    const int i = t / (ST * ST), j = (t / ST) % ST, k = t % ST;
+                // a thread's nodes share (j, k); tile node i lies in block (i + 3) / 4
+                // of the three along an axis, at (i + 3) % 4
+                const int j = (tid >> 3) & 7, k = tid & 7;
+                const int *sl_jk = S.slot_s[kc & 1] + ((j + 3) >> 2) * 3 + ((k + 3) >> 2);
+                const int l_jk = ((j + 3) & 3) * 4 + ((k + 3) & 3);
+#pragma unroll
+                for (int r = 0; r < ST3 / TPB; ++r) {
+                    const int i = (tid >> 6) + r * (TPB / 64);
                     const int q = tidx(i, j, k);
                     float mm, a0, a1, a2;
                     if (SCAT == 0) {
@@ -1041,15 +1143,16 @@ __global__ void __launch_bounds__(TPB, 512 / TPB) k_substep(Dev D, int gpar, int
                     // cleared for the next chunk as it is read
                     S.t.i[q] = 0; S.t.i[ST3P + q] = 0; S.t.i[2 * ST3P + q] = 0; S.t.i[3 * ST3P + q] = 0;
                     if (mm != 0.f) {
-                        const int I = ox - 1 + i, J = oy - 1 + j, K = oz - 1 + k;
-                        const int sl = S.slot_s[kc & 1][(((I >> 2) - bx + 1) * 3 + ((J >> 2) - by + 1)) * 3 +
-                                                        ((K >> 2) - bz + 1)];
-                        if (sl >= 0) red_add_v4(D.gmv[spar] + (size_t)sl * BLK_NODES + node_local(I, J, K), a0, a1, a2, mm);
-                        else set_err(D, ERRB_CAPACITY);
+                        const int sl = sl_jk[((i + 3) >> 2) * 9];
+                        if (sl >= 0)
+                            red_add_v4(D.gmv[spar] + (size_t)sl * BLK_NODES + ((i + 3) & 3) * 16 + l_jk, a0, a1, a2, mm);
+                        else
+                            set_err(D, ERRB_CAPACITY);
                     }
                 }
             }
         }
+        if (entry != NO_ENTRY) (DB ? D.occd[spar] : D.occ)[entry] = ticket.key;   // claimed before the flush
         // level 3 of chunk c + G has landed
         cp_async_wait_all();
         __syncthreads();
@@ -1134,39 +1237,48 @@ void launch_plan(const Dev &D, int bump_mask, cudaStream_t st) { k_plan<<<1, 102
 void launch_prepare(const Dev &D, int upd_par, int act_par, int do_sort, int keep_momentum, int grid, cudaStream_t st) {
     k_prepare<<<grid, 256, 0, st>>>(D, upd_par, act_par, do_sort, keep_momentum);
 }
-template <int MODE, int SCAT, int TPB, bool XM, bool DB = false>
-static void launch_sub(const Dev &D, int gpar, int spar, int grid, cudaStream_t st) {
-    k_substep<MODE, SCAT, TPB, XM, DB><<<grid, TPB, sizeof(SubstepSmem<TPB>), st>>>(D, gpar, spar);
+template <int MODE, int SCAT, int TPB, bool XM, bool DB = false, bool OWN = false>
+static void launch_sub(const Dev &D, int gpar, int spar, int grid, int keep, cudaStream_t st) {
+    k_substep<MODE, SCAT, TPB, XM, DB, OWN><<<grid, TPB, substep_smem<TPB, OWN>(), st>>>(D, gpar, spar, keep);
 }
 template <int TPB>
-static void launch_tpb(const Dev &D, int mode, int gpar, int spar, int grid, bool direct, cudaStream_t st) {
+static void launch_tpb(const Dev &D, int mode, int gpar, int spar, int grid, bool direct, int flags, cudaStream_t st) {
+    const int keep = flags & SUB_KEEP;
+    const bool own = (flags & SUB_OWN) != 0;
     if (direct && mode == MODE_FUSED) {   // direct binning: scatter strategies 1 and 2
-        if (D.xm) launch_sub<MODE_FUSED, 1, TPB, true, true>(D, gpar, spar, grid, st);
-        else if (D.scatter == 2) launch_sub<MODE_FUSED, 2, TPB, false, true>(D, gpar, spar, grid, st);
-        else launch_sub<MODE_FUSED, 1, TPB, false, true>(D, gpar, spar, grid, st);
+        if (D.xm) {
+            if (own) launch_sub<MODE_FUSED, 1, TPB, true, true, true>(D, gpar, spar, grid, keep, st);
+            else launch_sub<MODE_FUSED, 1, TPB, true, true>(D, gpar, spar, grid, keep, st);
+        } else if (D.scatter == 2) {
+            launch_sub<MODE_FUSED, 2, TPB, false, true>(D, gpar, spar, grid, keep, st);
+        } else if (own) {
+            launch_sub<MODE_FUSED, 1, TPB, false, true, true>(D, gpar, spar, grid, keep, st);
+        } else {
+            launch_sub<MODE_FUSED, 1, TPB, false, true>(D, gpar, spar, grid, keep, st);
+        }
         return;
     }
     if (D.xm) {   // further models: the shared-memory fixed-point scatter only
-        if (mode == MODE_G2P) launch_sub<MODE_G2P, 2, TPB, true>(D, gpar, spar, grid, st);
-        else if (mode == MODE_P2G) launch_sub<MODE_P2G, 1, TPB, true>(D, gpar, spar, grid, st);
-        else launch_sub<MODE_FUSED, 1, TPB, true>(D, gpar, spar, grid, st);
+        if (mode == MODE_G2P) launch_sub<MODE_G2P, 2, TPB, true>(D, gpar, spar, grid, keep, st);
+        else if (mode == MODE_P2G) launch_sub<MODE_P2G, 1, TPB, true>(D, gpar, spar, grid, keep, st);
+        else launch_sub<MODE_FUSED, 1, TPB, true>(D, gpar, spar, grid, keep, st);
         return;
     }
-    if (mode == MODE_G2P) { launch_sub<MODE_G2P, 2, TPB, false>(D, gpar, spar, grid, st); return; }
+    if (mode == MODE_G2P) { launch_sub<MODE_G2P, 2, TPB, false>(D, gpar, spar, grid, keep, st); return; }
     if (mode == MODE_P2G) {
-        if (D.scatter == 0) launch_sub<MODE_P2G, 0, TPB, false>(D, gpar, spar, grid, st);
-        else if (D.scatter == 1) launch_sub<MODE_P2G, 1, TPB, false>(D, gpar, spar, grid, st);
-        else launch_sub<MODE_P2G, 2, TPB, false>(D, gpar, spar, grid, st);
+        if (D.scatter == 0) launch_sub<MODE_P2G, 0, TPB, false>(D, gpar, spar, grid, keep, st);
+        else if (D.scatter == 1) launch_sub<MODE_P2G, 1, TPB, false>(D, gpar, spar, grid, keep, st);
+        else launch_sub<MODE_P2G, 2, TPB, false>(D, gpar, spar, grid, keep, st);
         return;
     }
-    if (D.scatter == 0) launch_sub<MODE_FUSED, 0, TPB, false>(D, gpar, spar, grid, st);
-    else if (D.scatter == 1) launch_sub<MODE_FUSED, 1, TPB, false>(D, gpar, spar, grid, st);
-    else launch_sub<MODE_FUSED, 2, TPB, false>(D, gpar, spar, grid, st);
+    if (D.scatter == 0) launch_sub<MODE_FUSED, 0, TPB, false>(D, gpar, spar, grid, keep, st);
+    else if (D.scatter == 1) launch_sub<MODE_FUSED, 1, TPB, false>(D, gpar, spar, grid, keep, st);
+    else launch_sub<MODE_FUSED, 2, TPB, false>(D, gpar, spar, grid, keep, st);
 }
 // the chunk size selects the CTA size: chunks of <= 64 particles run 64-thread CTAs
-void launch_substep(const Dev &D, int mode, int gpar, int spar, int grid, bool direct, cudaStream_t st) {
-    if (D.chunk <= 64) launch_tpb<64>(D, mode, gpar, spar, grid, direct, st);
-    else launch_tpb<128>(D, mode, gpar, spar, grid, direct, st);
+void launch_substep(const Dev &D, int mode, int gpar, int spar, int grid, bool direct, int flags, cudaStream_t st) {
+    if (D.chunk <= 64) launch_tpb<64>(D, mode, gpar, spar, grid, direct, flags, st);
+    else launch_tpb<128>(D, mode, gpar, spar, grid, direct, flags, st);
 }
 void launch_between(const Dev &D, int upd, int act, int grid, cudaStream_t st) {
     k_between<<<grid, 256, 0, st>>>(D, upd, act);
@@ -1179,13 +1291,16 @@ void launch_grid_dense(const Dev &D, int par, int which, float *m, float *mv, cu
 }
 template <int MODE, int SCAT, int TPB, bool XM> static int occ_of() {
     int nb = 0;
-    cudaFuncSetAttribute(k_substep<MODE, SCAT, TPB, XM, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)sizeof(SubstepSmem<TPB>));
-    if constexpr (MODE == MODE_FUSED && SCAT != 0)   // its direct-binning variant
-        cudaFuncSetAttribute(k_substep<MODE, SCAT, TPB, XM, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)sizeof(SubstepSmem<TPB>));
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_substep<MODE, SCAT, TPB, XM, false>, TPB,
-                                                  sizeof(SubstepSmem<TPB>));
+    cudaFuncSetAttribute(k_substep<MODE, SCAT, TPB, XM, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)substep_smem<TPB, false>());
+    if constexpr (MODE == MODE_FUSED && SCAT != 0)   // its direct-binning variants
+        cudaFuncSetAttribute(k_substep<MODE, SCAT, TPB, XM, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)substep_smem<TPB, false>());
+    if constexpr (MODE == MODE_FUSED && SCAT == 1)
+        cudaFuncSetAttribute(k_substep<MODE, SCAT, TPB, XM, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)substep_smem<TPB, true>());
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_substep<MODE, SCAT, TPB, XM, false, false>, TPB,
+                                                  substep_smem<TPB, false>());
     return nb;
 }
 template <int TPB> static int occ_tpb(int mode, int scatter, bool xm) {

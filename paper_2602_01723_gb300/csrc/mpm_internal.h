@@ -48,8 +48,11 @@ void launch_load(const Dev &D, const LoadArgs &a, cudaStream_t st);
 void launch_bin(const Dev &D, cudaStream_t st);
 void launch_plan(const Dev &D, int bump_mask, cudaStream_t st);
 void launch_prepare(const Dev &D, int upd_par, int act_par, int do_sort, int keep_momentum, int grid, cudaStream_t st);
+// flags of the fused mode: SUB_KEEP writes v and C to the records, SUB_OWN
+// (direct binning, fixed-point scatter) scatters in list order (see k_substep)
+enum { SUB_KEEP = 1, SUB_OWN = 2 };
 // direct: the fused mode bins straight into the scatter buffer's lists
-void launch_substep(const Dev &D, int mode, int gpar, int spar, int grid, bool direct, cudaStream_t st);
+void launch_substep(const Dev &D, int mode, int gpar, int spar, int grid, bool direct, int flags, cudaStream_t st);
 // between two direct-binning substeps: grid update of upd, work items of its
 // binning, activation of act (see k_between)
 void launch_between(const Dev &D, int upd, int act, int grid, cudaStream_t st);
@@ -150,11 +153,12 @@ struct mpm_ctx {
     bool trace_on = false;
     std::vector<cudaEvent_t> trace_ev[3];   // per substep mode: start, end, start, end, ...
     size_t trace_used[3] = {0, 0, 0};
-    // CUDA graph of two steady-state substeps (one per grid-buffer parity)
+    // CUDA graphs of steady-state substeps: [0] two (one per grid-buffer
+    // parity), [1] a whole reordering period of a direct-binning run
     bool use_graph = true;
-    cudaStream_t cap_stream = nullptr;   // library-owned stream the graph is captured on
-    cudaGraphExec_t graph2 = nullptr;
-    long long graph_key = -1;     // (n, buffer generation) the graph was captured for
+    cudaStream_t cap_stream = nullptr;   // library-owned stream the graphs are captured on
+    cudaGraphExec_t graph[2] = {nullptr, nullptr};
+    long long graph_key[2] = {-1, -1};   // (n, buffer generation, binning) each was captured for
     long long generation = 0;     // bumped whenever a device buffer the kernels use is reallocated
     bool bins_pending = false;    // a binning (counts / occupied list) awaits its plan
     // direct binning of the steady-state forward substeps: its lists are
@@ -183,7 +187,8 @@ void L_plan(mpm_ctx *ctx, int bump_mask, cudaStream_t st);
 void L_prepare(mpm_ctx *ctx, int upd_par, int act_par, int do_sort, cudaStream_t st, int keep_momentum = 0);
 // direct: bin straight into the scatter buffer's lists (fused mode); in_par
 // >= 0: read the work items of the direct binning into buffer in_par
-void L_substep(mpm_ctx *ctx, int mode, int gpar, int spar, cudaStream_t st, bool direct = false, int in_par = -1);
+void L_substep(mpm_ctx *ctx, int mode, int gpar, int spar, cudaStream_t st, bool direct = false, int in_par = -1,
+               int flags = SUB_KEEP);
 void L_between(mpm_ctx *ctx, int upd, int act, cudaStream_t st);
 void L_bin(mpm_ctx *ctx, cudaStream_t st);
 void launch_bgdo_accum(const Dev &D, const float4 *key, const float4 *post, int first, float inv_k,
