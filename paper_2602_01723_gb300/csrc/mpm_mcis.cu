@@ -8,9 +8,12 @@
 //   * surface points are binned per object into a uniform grid over the unit
 //     cube (App. C.1 normalises every scene to it; coordinates outside are
 //     clamped into the border cells, which keeps every pair within the
-//     cut-off in neighbouring cells) with a counting sort;
-//   * every candidate searches rings of cells in order of distance and stops
-//     once the best distance is below the ring's lower bound.  Beyond
+//     cut-off in neighbouring cells) with a counting sort.  The grid is kept as
+//     one occupancy bit per cell; occupied cells are numbered by their rank
+//     among the bits and carry their points' range and bounding box;
+//   * candidates are taken in cell order, a warp's worth of neighbours at a
+//     time, and search rings of cells in order of distance until the best
+//     distance is below the ring's lower bound.  Beyond
 //     d_cut = sigma sqrt(2 ln(1/eps)) the weight is eps whatever the
 //     distance, so the search radius is d_cut.  Distances are screened in
 //     FP32 and confirmed in FP64, so the minimum is the exact FP64 one;
@@ -19,6 +22,7 @@
 //     binary-searches its object's cumulative sums for floor(u W_k).
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -34,7 +38,7 @@ namespace {
 thread_local std::string g_mcis_msg;
 
 constexpr double WSCALE = 1099511627776.0;   // 2^40
-constexpr int RINGS = 6;                      // cell edge >= d_cut / 6: rings 0..6 cover d_cut
+constexpr int RINGS = 6;                      // coarse cell edge >= d_cut / 6: rings 0..6 cover d_cut
 
 __device__ __forceinline__ int find_range(const int64_t *off, int n, int64_t i) {
     int lo = 0, hi = n;   // off[lo] <= i < off[hi]
@@ -50,34 +54,90 @@ __device__ __forceinline__ int cell_of(float x, float inv_h, int G) {
     return c < 0 ? 0 : (c >= G ? G - 1 : c);
 }
 
+// The search radius d_cut spans RINGS coarse cells.  The cells the surface
+// points are binned into are `sub` times finer along each axis, so that few
+// points share one (see search).
 struct Grid {
     int G;            // cells per axis
     float inv_h;
-    long long cells;  // per object
+    int zwords;       // words of 32 cells per row of the occupancy mask
+    int sub;          // cells per coarse cell and axis
 };
-
-__global__ void k_mc_count(int n_obj, const int64_t *soff, const float *surf, Grid g, unsigned *cnt,
-                           unsigned *rank) {
-    const int64_t n = soff[n_obj];
-    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x) {
-        const int k = find_range(soff, n_obj, s);
-        const int cx = cell_of(surf[3 * s], g.inv_h, g.G), cy = cell_of(surf[3 * s + 1], g.inv_h, g.G),
-                  cz = cell_of(surf[3 * s + 2], g.inv_h, g.G);
-        const long long key = (long long)k * g.cells + ((long long)cx * g.G + cy) * g.G + cz;
-        rank[s] = atomicAdd(&cnt[key], 1u);
-    }
+// occupied cells as the search reads them: one bit per cell, zwords per
+// (object, x, y) row, the last of a row always zero, so that any window of up to
+// 32 cells of a row lies in two consecutive words; per word the number
+// of occupied cells before it; per occupied cell (in that order) the box of its
+// points with their first index (lo.w) and number (hi.w)
+struct Cells {
+    const unsigned *mask, *before;
+    const float4 *lo, *hi;
+    const float4 *point;   // surface points by cell
+};
+__device__ __forceinline__ long long mask_row(const Grid &g, int k, int x, int y) {
+    return (((long long)k * g.G + x) * g.G + y) * g.zwords;
 }
 
-__global__ void k_mc_scatter(int n_obj, const int64_t *soff, const float *surf, Grid g, const unsigned *start,
-                             const unsigned *rank, float4 *sorted) {
+// unsigned integers that order like the floats they come from
+__device__ __forceinline__ unsigned ordered(float x) {
+    const unsigned u = __float_as_uint(x);
+    return (u & 0x80000000u) ? ~u : u | 0x80000000u;
+}
+__device__ __forceinline__ float unordered(unsigned u) {
+    return __uint_as_float((u & 0x80000000u) ? u & 0x7fffffffu : ~u);
+}
+
+// word and bit of a surface point's cell
+__device__ __forceinline__ long long point_word(int n_obj, const int64_t *soff, const float *surf, const Grid &g,
+                                                int64_t s, unsigned &bit) {
+    const int k = find_range(soff, n_obj, s);
+    const int cx = cell_of(surf[3 * s], g.inv_h, g.G), cy = cell_of(surf[3 * s + 1], g.inv_h, g.G),
+              cz = cell_of(surf[3 * s + 2], g.inv_h, g.G);
+    bit = 1u << (cz & 31);
+    return mask_row(g, k, cx, cy) + (cz >> 5);
+}
+
+__global__ void k_mc_mark(int n_obj, const int64_t *soff, const float *surf, Grid g, unsigned *mask) {
     const int64_t n = soff[n_obj];
     for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x) {
-        const int k = find_range(soff, n_obj, s);
-        const float x = surf[3 * s], y = surf[3 * s + 1], z = surf[3 * s + 2];
-        const long long key =
-            (long long)k * g.cells +
-            ((long long)cell_of(x, g.inv_h, g.G) * g.G + cell_of(y, g.inv_h, g.G)) * g.G + cell_of(z, g.inv_h, g.G);
-        sorted[start[key] + rank[s]] = make_float4(x, y, z, 0.f);
+        unsigned bit;
+        const long long w = point_word(n_obj, soff, surf, g, s, bit);
+        atomicOr(&mask[w], bit);
+    }
+}
+__global__ void k_mc_bits(const unsigned *mask, long long words, unsigned *bits) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < words; i += (long long)gridDim.x * blockDim.x)
+        bits[i] = __popc(mask[i]);
+}
+// points per occupied cell, each point's cell and rank in it, and the cells'
+// boxes (box: min xyz, max xyz as ordered integers, the minima complemented)
+__global__ void k_mc_count(int n_obj, const int64_t *soff, const float *surf, Grid g, const unsigned *mask,
+                           const unsigned *before, unsigned *cnt, unsigned *cell, unsigned *rank, unsigned *box) {
+    const int64_t n = soff[n_obj];
+    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x) {
+        unsigned bit;
+        const long long w = point_word(n_obj, soff, surf, g, s, bit);
+        const unsigned c = before[w] + __popc(mask[w] & (bit - 1u));
+        cell[s] = c;
+        rank[s] = atomicAdd(&cnt[c], 1u);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const unsigned u = ordered(surf[3 * s + a]);
+            atomicMax(&box[6 * (size_t)c + a], ~u);
+            atomicMax(&box[6 * (size_t)c + 3 + a], u);
+        }
+    }
+}
+__global__ void k_mc_scatter(int64_t n, const float *surf, const unsigned *start, const unsigned *cell,
+                             const unsigned *rank, const unsigned *cnt, const unsigned *box, float4 *sorted,
+                             float4 *lo, float4 *hi) {
+    for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x) {
+        const unsigned c = cell[s], r = rank[s], s0 = start[c];
+        sorted[s0 + r] = make_float4(surf[3 * s], surf[3 * s + 1], surf[3 * s + 2], 0.f);
+        if (r == 0) {   // one point per cell writes its box
+            const unsigned *b = box + 6 * (size_t)c;
+            lo[c] = make_float4(unordered(~b[0]), unordered(~b[1]), unordered(~b[2]), __uint_as_float(s0));
+            hi[c] = make_float4(unordered(b[3]), unordered(b[4]), unordered(b[5]), __uint_as_float(cnt[c]));
+        }
     }
 }
 
@@ -143,31 +203,25 @@ __global__ void k_mc_scan_i64_add(long long *out, long long n, const long long *
     if (i < n) out[i] += totals[blockIdx.x];
 }
 
-// candidates in (object, cell) order, so that the threads of a warp search
-// the same cells
-__global__ void k_mc_cand_count(int n_obj, const int64_t *coff, const float *cand, Grid g, unsigned *cnt,
-                                unsigned *rank) {
+// candidates in (object, cell) order of a grid of G cells per axis, so that the
+// candidates of a warp are neighbours
+__global__ void k_mc_cand_count(int n_obj, const int64_t *coff, const float *cand, int G, unsigned *cnt,
+                                unsigned *cell, unsigned *rank) {
     const int64_t n = coff[n_obj];
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
         const int k = find_range(coff, n_obj, j);
-        const long long key = (long long)k * g.cells +
-                              ((long long)cell_of(cand[3 * j], g.inv_h, g.G) * g.G + cell_of(cand[3 * j + 1], g.inv_h, g.G)) *
-                                  g.G + cell_of(cand[3 * j + 2], g.inv_h, g.G);
+        const float ih = (float)G;
+        const unsigned key = (unsigned)((((long long)k * G + cell_of(cand[3 * j], ih, G)) * G + cell_of(cand[3 * j + 1], ih, G)) * G +
+                                        cell_of(cand[3 * j + 2], ih, G));
+        cell[j] = key;
         rank[j] = atomicAdd(&cnt[key], 1u);
     }
 }
-__global__ void k_mc_cand_scatter(int n_obj, const int64_t *coff, const float *cand, Grid g, const unsigned *start,
-                                  const unsigned *rank, unsigned *order) {
-    const int64_t n = coff[n_obj];
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
-        const int k = find_range(coff, n_obj, j);
-        const long long key = (long long)k * g.cells +
-                              ((long long)cell_of(cand[3 * j], g.inv_h, g.G) * g.G + cell_of(cand[3 * j + 1], g.inv_h, g.G)) *
-                                  g.G + cell_of(cand[3 * j + 2], g.inv_h, g.G);
-        order[start[key] + rank[j]] = (unsigned)j;
-    }
+__global__ void k_mc_cand_scatter(int64_t n, const unsigned *start, const unsigned *cell, const unsigned *rank,
+                                  unsigned *order) {
+    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x)
+        order[start[cell[j]] + rank[j]] = (unsigned)j;
 }
-
 
 // squared distance along one axis from q to cell c of edge h, in FP32
 __device__ __forceinline__ float box_d2f(float q, int c, float h) {
@@ -176,58 +230,75 @@ __device__ __forceinline__ float box_d2f(float q, int c, float h) {
     return e * e;
 }
 
-// steps 1 and 2 per candidate: exact nearest-surface distance within d_cut, weight
-__global__ void k_mc_nn(int n_obj, const int64_t *coff, const float *cand, const unsigned *order, Grid g,
-                        const unsigned *start, const unsigned *cnt, const float4 *sorted, double sigma, double eps,
-                        double *d, double *w, long long *wq) {
-    const int64_t n = coff[n_obj];
-    const double h = 1.0 / (double)g.inv_h;
-    const float hf = 1.f / g.inv_h;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t j = order[t];
-        const int k = find_range(coff, n_obj, j);
-        const float qx = cand[3 * j], qy = cand[3 * j + 1], qz = cand[3 * j + 2];
-        const int cx = cell_of(qx, g.inv_h, g.G), cy = cell_of(qy, g.inv_h, g.G), cz = cell_of(qz, g.inv_h, g.G);
-        const long long base = (long long)k * g.cells;
-        double best = INFINITY;
-        float screen = INFINITY;   // best * (1 + 1e-6), rounded up to FP32
-        for (int r = 0; r <= RINGS; ++r) {
-            // cells of ring r lie at least (r - 1) h away: stop once the best is closer
-            const double lb = (double)(r - 1) * h;
-            if (r > 1 && best <= lb * lb) break;
-            // pruning threshold in FP32: the FP32 box distance of a cell within d_cut is
-            // within 1.3e-7 of the exact one (cell edges and differences rounded), so this
-            // margin never skips a cell that could hold a closer point
-            const float prune = (float)best * 1.00001f + 2e-7f;
-            for (int ix = -r; ix <= r; ++ix) {
-                const int x = cx + ix;
-                if (x < 0 || x >= g.G) continue;
-                for (int iy = -r; iy <= r; ++iy) {
-                    const int y = cy + iy;
-                    if (y < 0 || y >= g.G) continue;
-                    // ring r only: the whole row on its x or y faces, else its two z ends
-                    const bool face = ix == -r || ix == r || iy == -r || iy == r;
-                    const int zstep = (face || r == 0) ? 1 : 2 * r;
-                    for (int iz = -r; iz <= r; iz += zstep) {
-                        const int z = cz + iz;
-                        if (z < 0 || z >= g.G) continue;
-                        // a cell wholly farther than the best point holds nothing closer
-                        // (cells are clamped at the cube's faces, so only interior cells are skipped)
-                        if (x > 0 && y > 0 && z > 0 && x < g.G - 1 && y < g.G - 1 && z < g.G - 1 &&
-                            box_d2f(qx, x, hf) + box_d2f(qy, y, hf) + box_d2f(qz, z, hf) > prune)
-                            continue;
-                        const long long key = base + ((long long)x * g.G + y) * g.G + z;
-                        const unsigned s0 = start[key], s1 = s0 + cnt[key];
+// ... from q to the range [lo, hi], and from [a, b] to it
+__device__ __forceinline__ float range_d2f(float q, float lo, float hi) {
+    const float e = fmaxf(0.f, fmaxf(lo - q, q - hi));
+    return e * e;
+}
+__device__ __forceinline__ float gap2(float a, float b, float lo, float hi) {
+    const float e = fmaxf(0.f, fmaxf(lo - b, a - hi));
+    return e * e;
+}
+
+__device__ __forceinline__ double dist2(float qx, float qy, float qz, float4 c) {
+    const double fx = (double)qx - (double)c.x, fy = (double)qy - (double)c.y, fz = (double)qz - (double)c.z;
+    return fx * fx + fy * fy + fz * fz;
+}
+
+// Squared distance to the nearest surface point in the coarse cells up to RINGS
+// away, every decision in FP64; one thread.  For a candidate with nothing
+// within d_cut (the coarse cells then say how far it looked), or whose three
+// nearest points agree to FP32 rounding (repeated points).
+__device__ __noinline__ double nn_exact(float qx, float qy, float qz, int k, const Grid &g, const Cells &C) {
+    const int Gc = g.G / g.sub;
+    const float inv_hc = g.inv_h / (float)g.sub;
+    const double h = 1.0 / (double)inv_hc;
+    const float hf = 1.f / inv_hc;
+    const int cx = cell_of(qx, inv_hc, Gc), cy = cell_of(qy, inv_hc, Gc), cz = cell_of(qz, inv_hc, Gc);
+    double best = INFINITY;
+    float screen = INFINITY;   // best * (1 + 1e-6), rounded up to FP32
+    for (int r = 0; r <= RINGS; ++r) {
+        // cells of ring r lie at least (r - 1) h away: stop once the best is closer
+        const double lb = (double)(r - 1) * h;
+        if (r > 1 && best <= lb * lb) break;
+        // pruning threshold in FP32: the FP32 box distance of a cell within d_cut is
+        // within 1.3e-7 of the exact one (cell edges and differences rounded), so this
+        // margin never skips a cell that could hold a closer point
+        const float prune = (float)best * 1.00001f + 2e-7f;
+        for (int ix = -r; ix <= r; ++ix) {
+            const int x = cx + ix;
+            if (x < 0 || x >= Gc) continue;
+            for (int iy = -r; iy <= r; ++iy) {
+                const int y = cy + iy;
+                if (y < 0 || y >= Gc) continue;
+                // ring r only: the whole row on its x or y faces, else its two z ends
+                const bool face = ix == -r || ix == r || iy == -r || iy == r;
+                const int zstep = (face || r == 0) ? 1 : 2 * r;
+                for (int iz = -r; iz <= r; iz += zstep) {
+                    const int z = cz + iz;
+                    if (z < 0 || z >= Gc) continue;
+                    // a cell wholly farther than the best point holds nothing closer
+                    // (cells are clamped at the cube's faces, so only interior cells are skipped)
+                    if (x > 0 && y > 0 && z > 0 && x < Gc - 1 && y < Gc - 1 && z < Gc - 1 &&
+                        box_d2f(qx, x, hf) + box_d2f(qy, y, hf) + box_d2f(qz, z, hf) > prune)
+                        continue;
+                    for (int a = 0; a < g.sub * g.sub * g.sub; ++a) {   // its cells
+                        const int fz = z * g.sub + a % g.sub, fy = y * g.sub + a / g.sub % g.sub, fx = x * g.sub + a / (g.sub * g.sub);
+                        const long long w = mask_row(g, k, fx, fy) + (fz >> 5);
+                        const unsigned word = C.mask[w], bit = 1u << (fz & 31);
+                        if (!(word & bit)) continue;
+                        const unsigned c = C.before[w] + __popc(word & (bit - 1u));
+                        const float4 lo = C.lo[c], hi = C.hi[c];
+                        if (range_d2f(qx, lo.x, hi.x) + range_d2f(qy, lo.y, hi.y) + range_d2f(qz, lo.z, hi.z) > prune) continue;
+                        const unsigned s0 = __float_as_uint(lo.w), s1 = s0 + __float_as_uint(hi.w);
                         for (unsigned s = s0; s < s1; ++s) {
-                            const float4 c = sorted[s];
-                            const float ex = qx - c.x, ey = qy - c.y, ez = qz - c.z;
+                            const float4 t = C.point[s];
+                            const float ex = qx - t.x, ey = qy - t.y, ez = qz - t.z;
                             const float d2f = ex * ex + ey * ey + ez * ez;
                             // the FP32 value is within 1e-6 relative of the exact one, so a
                             // point closer than best passes this FP32 screen
                             if (d2f <= screen) {
-                                const double fx = (double)qx - (double)c.x, fy = (double)qy - (double)c.y,
-                                             fz = (double)qz - (double)c.z;
-                                const double d2 = fx * fx + fy * fy + fz * fz;
+                                const double d2 = dist2(qx, qy, qz, t);
                                 if (d2 < best) {
                                     best = d2;
                                     screen = __double2float_ru(best * (1.0 + 1e-6));
@@ -238,6 +309,450 @@ __global__ void k_mc_nn(int n_obj, const int64_t *coff, const float *cand, const
                 }
             }
         }
+    }
+    return best;
+}
+
+// the three smallest FP32 squared distances seen, with the points of the two
+// smallest; a NaN is never kept
+struct Near3 {
+    float d1, d2, d3;
+    unsigned i1, i2;
+    __device__ __forceinline__ void clear() {
+        d1 = d2 = d3 = INFINITY;
+        i1 = i2 = 0;
+    }
+    __device__ __forceinline__ void add(float d, unsigned i) {
+        if (!(d < d3)) return;
+        if (d < d1) {
+            d3 = d2; d2 = d1; i2 = i1;
+            d1 = d; i1 = i;
+        } else if (d < d2) {
+            d3 = d2;
+            d2 = d; i2 = i;
+        } else {
+            d3 = d;
+        }
+    }
+};
+
+__device__ __forceinline__ unsigned lanes_before() {
+    unsigned m;
+    asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
+    return m;
+}
+// the i-th lowest lane of a mask
+__device__ __forceinline__ int nth_lane(unsigned lanes, int i) { return (int)__fns(lanes, 0, i + 1); }
+
+// warp minimum and maximum of non-negative floats (their bit patterns order alike)
+__device__ __forceinline__ float warp_min(float x) {
+    return __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(x)));
+}
+__device__ __forceinline__ float warp_max(float x) {
+    return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(x)));
+}
+
+// A group of candidates that search together: the cells they lie in and their
+// bounding box
+struct Group {
+    int k;                 // object
+    int c0[3], c1[3];      // cells
+    float a[3], b[3];      // box
+};
+
+constexpr int NN_WARPS = 4;        // warps per CTA of the search
+constexpr int TURN = 8;            // candidates a warp takes at a time, four lanes each
+constexpr int FIRST_RINGS = 2;     // reach of the first pass, unless the first bound is
+constexpr int DIRECT_RINGS = 4;    // this close already
+constexpr int SAMPLES = 8;         // surface points each lane tries for a first bound
+struct WarpScratch {
+    unsigned cell[1024];           // occupied cells still to be read: mask word << 5 | bit
+    float4 pt[32];                 // points (x y z, index) that every candidate meets
+    float two[TURN / 2][8];        // candidates 2 u, 2 u + 1: x x y y z z, bounds
+    unsigned char order[32];       // candidates by (cell, octant of the cell)
+};
+
+// packed pairs of FP32 operations, one instruction each
+__device__ __forceinline__ unsigned long long pack2(float2 a) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a.x), "f"(a.y));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long a) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a));
+    return r;
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
+    return unpack2(r);
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+    unsigned long long r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
+    return unpack2(r);
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)), "l"(pack2(c)));
+    return unpack2(r);
+}
+// distances from two coordinates to the range [lo, -nhi]
+__device__ __forceinline__ float2 range_pair(float2 q, float lo, float nhi) {
+    const float2 over = add2(q, make_float2(nhi, nhi));
+    return make_float2(fmaxf(0.f, fmaxf(lo - q.x, over.x)), fmaxf(0.f, fmaxf(lo - q.y, over.y)));
+}
+
+// Distances from the lanes' candidates to the points of the cells of the lanes
+// in `keep` (lane l: points s0 .. s0 + n), read 32 at a time.  BY_POINT: one
+// candidate, each lane takes a point; otherwise the four lanes of a candidate
+// take a quarter each, passed through shared memory.
+template <bool BY_POINT>
+__device__ __forceinline__ void meet(Near3 &m, float qx, float qy, float qz, unsigned keep, unsigned s0, unsigned n,
+                                     const float4 *sorted, WarpScratch &W) {
+    const int lane = threadIdx.x & 31;
+    const unsigned mine = (keep >> lane) & 1u ? n : 0u;
+    unsigned incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned u = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += u;
+    }
+    const unsigned first = s0 - (incl - mine);   // point of running index i in this lane's cell: first + i
+    const unsigned total = __shfl_sync(0xffffffffu, incl, 31);
+    for (unsigned p0 = 0; p0 < total; p0 += 32) {
+        const unsigned i = p0 + lane;
+        int c = 0;   // the cell that holds running index i
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+            if (__shfl_sync(0xffffffffu, incl, c + o - 1) <= i) c += o;
+        const unsigned s = __shfl_sync(0xffffffffu, first, c & 31) + i;
+        if (BY_POINT) {
+            if (i < total) {
+                const float4 t = sorted[s];
+                const float ex = qx - t.x, ey = qy - t.y, ez = qz - t.z;
+                m.add(ex * ex + ey * ey + ez * ez, s);
+            }
+        } else {
+            __syncwarp();
+            if (i < total) {
+                float4 t = sorted[s];
+                t.w = __uint_as_float(s);
+                W.pt[lane] = t;
+            }
+            __syncwarp();
+            const int cnt = (int)min(32u, total - p0);
+#pragma unroll 4
+            for (int u = lane & 3; u < cnt; u += 4) {
+                const float4 t = W.pt[u];
+                const float ex = qx - t.x, ey = qy - t.y, ez = qz - t.z;
+                m.add(ex * ex + ey * ey + ez * ez, __float_as_uint(t.w));
+            }
+        }
+    }
+}
+
+// Searches the cells around a group for the nearest surface points within
+// sqrt(cut2).  BY_POINT: one candidate for the whole warp; otherwise one per
+// four lanes, where they are active.  seed: a squared distance that the
+// candidate's nearest point is known not to exceed (INFINITY: none).  The whole warp calls it, and
+// all of its memory accesses are made 32 at a time: the lanes look up one row
+// of cells each in the occupancy mask, then the box of one occupied cell each,
+// then one point each.  A pass takes the cells up to R away from the group's;
+// a second one, over the rest, follows where R proved too small.  Cells are
+// dropped whose points are farther than the best point so far of every
+// candidate; the first to be read is the one closest to the group.
+template <bool BY_POINT>
+__device__ __forceinline__ void search(Near3 &m, bool active, float qx, float qy, float qz, float seed, const Group &p,
+                                       float cut2, const Grid &g, const Cells &C, WarpScratch &W) {
+    const int lane = threadIdx.x & 31;
+    const float hf = 1.f / g.inv_h;
+    seed = fminf(seed, cut2);
+    auto bound = [&]() {   // squared distance beyond which no candidate needs a point, with the margin of FP32 box distances
+        seed = fminf(seed, m.d1);
+        if (!BY_POINT) {
+            seed = fminf(seed, __shfl_xor_sync(0xffffffffu, seed, 1));
+            seed = fminf(seed, __shfl_xor_sync(0xffffffffu, seed, 2));
+        }
+        return (BY_POINT ? warp_min(seed) : warp_max(active ? seed : 0.f)) * 1.00001f + 2e-7f;
+    };
+    // cells more than R away lie at least R h away; R_most h is past the
+    // cut-off (or past the grid), which keeps a window of z cells below 32
+    const int R_most = min(RINGS * g.sub + 2, g.G);
+    float worst = bound();
+    auto rings = [&](int least) {
+        const float x = sqrtf(worst) * g.inv_h;
+        return x < (float)R_most ? max(least, (int)x + 1) : R_most;
+    };
+    bool seeded = false;
+    int done = -1;   // cells up to this far away have been taken
+    for (int R = rings(1) <= DIRECT_RINGS ? rings(1) : FIRST_RINGS;;) {
+        const int X0 = p.c0[0] - R, Y0 = p.c0[1] - R, X1 = p.c1[0] + R, Y1 = p.c1[1] + R;
+        const int wy = Y1 - Y0 + 1, rows = (X1 - X0 + 1) * wy;
+        const int z0 = max(p.c0[2] - R, 0), z1 = min(p.c1[2] + R, g.G - 1);
+        const unsigned all = 0xffffffffu >> (31 - (z1 - z0));
+        // the window's cells that an earlier pass took, in the rows it took
+        const int d0 = max(p.c0[2] - done, 0), d1 = min(p.c1[2] + done, g.G - 1);
+        const unsigned old = done < 0 ? 0u : (0xffffffffu >> (31 - (d1 - d0))) << (d0 - z0);
+        const float iw = 1.f / (float)wy;
+        int listed = 0;   // cells in the list
+        for (int c0 = 0; c0 < rows; c0 += 32) {
+            const int c = c0 + lane;
+            const int ix = (int)(((float)c + 0.5f) * iw);   // c / wy: c < 2^10, never near an integer
+            const int x = X0 + ix, y = Y0 + c - ix * wy;
+            unsigned bits = 0;             // occupied cells z0 .. z1 of the row that belong to this pass
+            unsigned at = 0;               // of z0's cell: mask word << 5 | bit
+            // a row at the cube's face also holds what lies beyond it and is always looked up
+            if (c < rows && x >= 0 && y >= 0 && x < g.G && y < g.G &&
+                (x == 0 || y == 0 || x == g.G - 1 || y == g.G - 1 ||
+                 gap2(p.a[0], p.b[0], (float)x * hf, (float)(x + 1) * hf) +
+                         gap2(p.a[1], p.b[1], (float)y * hf, (float)(y + 1) * hf) <= worst)) {
+                const long long row = mask_row(g, p.k, x, y) + (z0 >> 5);
+                at = (unsigned)row << 5 | (z0 & 31);
+                bits = __funnelshift_r(C.mask[row], C.mask[row + 1], z0 & 31) & all;
+                if (x >= p.c0[0] - done && x <= p.c1[0] + done && y >= p.c0[1] - done && y <= p.c1[1] + done) bits &= ~old;
+            }
+            if (__any_sync(0xffffffffu, bits != 0)) {
+                unsigned incl = __popc(bits);
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const unsigned u = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += u;
+                }
+                __syncwarp();
+                for (int to = listed + (int)incl - __popc(bits); bits; bits &= bits - 1)
+                    W.cell[to++] = at + (unsigned)(__ffs(bits) - 1);
+                listed += (int)__shfl_sync(0xffffffffu, incl, 31);
+                __syncwarp();
+            }
+            // 32 cells at a time, what is left over after the last row
+            const bool last = c0 + 32 >= rows;
+            while (listed >= 32 || (last && listed > 0)) {
+                const int take = min(listed, 32);
+                listed -= take;
+                float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
+                float dist = INFINITY;
+                if (lane < take) {
+                    const unsigned e = W.cell[listed + lane];
+                    const unsigned c = C.before[e >> 5] + __popc(C.mask[e >> 5] & ((1u << (e & 31)) - 1u));
+                    lo = C.lo[c];
+                    hi = C.hi[c];
+                    dist = gap2(p.a[0], p.b[0], lo.x, hi.x) + gap2(p.a[1], p.b[1], lo.y, hi.y) +
+                           gap2(p.a[2], p.b[2], lo.z, hi.z);
+                }
+                worst = bound();
+                unsigned keep = __ballot_sync(0xffffffffu, dist <= worst);
+                if (!keep) continue;
+                const unsigned s0 = __float_as_uint(lo.w), n = __float_as_uint(hi.w);
+                if (!seeded) {
+                    // the closest cell first: its points bound what else is needed
+                    const unsigned near = __reduce_min_sync(0xffffffffu, __float_as_uint(dist));
+                    const unsigned one = __ballot_sync(0xffffffffu, __float_as_uint(dist) == near);
+                    const unsigned lead = one & (0u - one);
+                    meet<BY_POINT>(m, qx, qy, qz, lead, s0, n, C.point, W);
+                    worst = bound();
+                    keep = __ballot_sync(0xffffffffu, dist <= worst) & ~lead;
+                    seeded = true;
+                }
+                if (!BY_POINT && keep) {
+                    // the cells that some candidate of the group still needs:
+                    // each lane holds its cell against all candidates
+                    // (two candidates at a time in packed arithmetic)
+                    __syncwarp();
+                    if ((lane & 3) == 0) {
+                        float *o = &W.two[lane >> 3][(lane >> 2) & 1];
+                        o[0] = qx; o[2] = qy; o[4] = qz;
+                        o[6] = active ? seed * 1.00001f + 2e-7f : -1.f;
+                    }
+                    __syncwarp();
+                    const float nhx = -hi.x, nhy = -hi.y, nhz = -hi.z;
+                    bool want = false;
+#pragma unroll
+                    for (int u = 0; u < TURN / 2; ++u) {
+                        const float4 xy = *reinterpret_cast<const float4 *>(&W.two[u][0]);
+                        const float4 zb = *reinterpret_cast<const float4 *>(&W.two[u][4]);
+                        float2 e = range_pair(make_float2(xy.x, xy.y), lo.x, nhx);
+                        float2 acc = mul2(e, e);
+                        e = range_pair(make_float2(xy.z, xy.w), lo.y, nhy);
+                        acc = fma2(e, e, acc);
+                        e = range_pair(make_float2(zb.x, zb.y), lo.z, nhz);
+                        acc = fma2(e, e, acc);
+                        want |= acc.x <= zb.z || acc.y <= zb.w;
+                    }
+                    keep &= __ballot_sync(0xffffffffu, want);
+                }
+                if (keep) meet<BY_POINT>(m, qx, qy, qz, keep, s0, n, C.point, W);
+            }
+        }
+        worst = bound();
+        const float far = (float)R * hf;
+        if (R >= R_most || worst <= far * far) break;
+        done = R;
+        R = rings(R + 1);
+    }
+}
+
+// step 1 per candidate: exact squared distance to the nearest surface point
+// within d_cut.  A CTA takes NN_WARPS x per consecutive candidates in (object, cell)
+// order, orders them further by the octant of their cell, and each warp takes
+// `per` of them: those within `reach` cells of the first one search together,
+// four lanes each, when there are at least GROUP, else the first one alone with
+// the lanes on the points.  Distances are compared in FP32, whose value is
+// within 1e-6 relative of the exact one; the points that FP32 cannot tell apart
+// from the nearest (mostly none besides it) are settled in FP64.
+//
+// What bounds it: issue slots and the latency of three dependent loads per 32
+// cells (mask word, box, points).  750k candidates against 108k surface points:
+// 4.2 ms -> 0.76 ms; a thread per candidate walking the same cells took 2.4 ms
+// (divergent), 32 candidates of one lane each 1.3 ms (a few deep groups, whose
+// points are nearly equidistant, ran twice as long as all others).
+constexpr int GROUP = 2;
+__global__ void __launch_bounds__(32 * NN_WARPS) k_mc_nn(int n_obj, const int64_t *soff, const int64_t *coff,
+                                                         const float *cand, const unsigned *order, Grid g, Cells C,
+                                                         int per, int reach, float cells_sorted, float cut2,
+                                                         double *d2) {
+    __shared__ WarpScratch scratch[NN_WARPS];
+    WarpScratch &W = scratch[threadIdx.x >> 5];
+    const int64_t n = coff[n_obj];
+    const int lane = threadIdx.x & 31;
+    const int64_t t0 = (int64_t)blockIdx.x * NN_WARPS * per;
+    // the CTA's candidates (every warp looks at all of them), ordered within
+    // their cell by octant
+    float qx = 0.f, qy = 0.f, qz = 0.f;
+    int64_t j = -1;
+    int k = -1;
+    {
+        const bool in = lane < NN_WARPS * per && t0 + lane < n;
+        unsigned cell = 0xffffffffu, octant = 0;
+        if (in) {
+            j = order[t0 + lane];
+            k = find_range(coff, n_obj, j);
+            qx = cand[3 * j]; qy = cand[3 * j + 1]; qz = cand[3 * j + 2];
+            const float ux = qx * cells_sorted, uy = qy * cells_sorted, uz = qz * cells_sorted;
+            // candidates of one cell are side by side: any label of the cell does
+            cell = ((unsigned)(int)floorf(ux) * 73856093u ^ (unsigned)(int)floorf(uy) * 19349663u ^
+                    (unsigned)(int)floorf(uz) * 83492791u) & 0x7fffffffu;
+            octant = (ux - floorf(ux) >= 0.5f ? 1u : 0u) | (uy - floorf(uy) >= 0.5f ? 2u : 0u) |
+                     (uz - floorf(uz) >= 0.5f ? 4u : 0u);
+        }
+        const unsigned peers = __match_any_sync(0xffffffffu, cell);
+        int rank = 0;   // among the candidates of the cell, by (octant, lane)
+#pragma unroll
+        for (unsigned o = 0; o < 8; ++o) {
+            const unsigned m = __ballot_sync(0xffffffffu, octant == o) & peers;
+            if (o < octant) rank += __popc(m);
+            if (o == octant) rank += __popc(m & lanes_before());
+        }
+        const int to = nth_lane(peers, rank);
+        W.order[to] = (unsigned char)lane;
+        __syncwarp();
+        const int from = W.order[min(31, (threadIdx.x >> 5) * per + (lane >> 2))];
+        qx = __shfl_sync(0xffffffffu, qx, from);
+        qy = __shfl_sync(0xffffffffu, qy, from);
+        qz = __shfl_sync(0xffffffffu, qz, from);
+        j = __shfl_sync(0xffffffffu, j, from);
+        k = __shfl_sync(0xffffffffu, k, from);
+    }
+    const bool mine = (lane >> 2) < per && k >= 0;
+    const int cx = cell_of(qx, g.inv_h, g.G), cy = cell_of(qy, g.inv_h, g.G), cz = cell_of(qz, g.inv_h, g.G);
+    double best = INFINITY;
+    unsigned todo = __ballot_sync(0xffffffffu, mine);   // four bits per candidate
+    while (todo) {
+        const int lead = __ffs(todo) - 1;
+        Group p;
+        p.k = __shfl_sync(0xffffffffu, k, lead);
+        const int lx = __shfl_sync(0xffffffffu, cx, lead), ly = __shfl_sync(0xffffffffu, cy, lead),
+                  lz = __shfl_sync(0xffffffffu, cz, lead);
+        const float lqx = __shfl_sync(0xffffffffu, qx, lead), lqy = __shfl_sync(0xffffffffu, qy, lead),
+                    lqz = __shfl_sync(0xffffffffu, qz, lead);
+        const bool near_lead = k == p.k && abs(cx - lx) <= reach && abs(cy - ly) <= reach && abs(cz - lz) <= reach;
+        const unsigned same = __ballot_sync(0xffffffffu, near_lead) & todo;
+        const bool together = __popc(same) >= 4 * GROUP;
+        // a first bound: the closest to the first candidate of a few surface
+        // points spread over the object's cells
+        float seed = INFINITY;
+        const int64_t s_lo = soff[p.k], s_n = soff[p.k + 1] - s_lo;
+        if (s_n > 0) {
+            float near = INFINITY;
+            float4 at = make_float4(INFINITY, INFINITY, INFINITY, 0.f);
+#pragma unroll
+            for (int u = 0; u < SAMPLES; ++u) {
+                const float4 t = C.point[s_lo + (s_n * (u * 32 + lane)) / (32 * SAMPLES)];
+                const float ex = lqx - t.x, ey = lqy - t.y, ez = lqz - t.z;
+                const float e2 = ex * ex + ey * ey + ez * ez;
+                if (e2 < near) { near = e2; at = t; }
+            }
+            const unsigned who = __ballot_sync(0xffffffffu, near == warp_min(near));
+            const int src = __ffs(who) - 1;
+            const float ex = qx - __shfl_sync(0xffffffffu, at.x, src), ey = qy - __shfl_sync(0xffffffffu, at.y, src),
+                        ez = qz - __shfl_sync(0xffffffffu, at.z, src);
+            seed = ex * ex + ey * ey + ez * ez;
+            if (!(seed < INFINITY)) seed = INFINITY;   // nothing finite to go by
+        }
+        Near3 m;
+        m.clear();
+        float px = qx, py = qy, pz = qz;
+        bool active = (same >> lane) & 1u;
+        if (together) {
+            todo &= ~same;
+            if (!active) m.d3 = -1.f;   // keeps nothing
+            const int cc[3] = {cx, cy, cz}, lc[3] = {lx, ly, lz};
+            const float q[3] = {qx, qy, qz}, lq[3] = {lqx, lqy, lqz};
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                p.c0[a] = __reduce_min_sync(0xffffffffu, active ? cc[a] : lc[a]);
+                p.c1[a] = __reduce_max_sync(0xffffffffu, active ? cc[a] : lc[a]);
+                p.a[a] = unordered(__reduce_min_sync(0xffffffffu, ordered(active ? q[a] : lq[a])));
+                p.b[a] = unordered(__reduce_max_sync(0xffffffffu, ordered(active ? q[a] : lq[a])));
+            }
+            search<false>(m, active, px, py, pz, seed, p, cut2, g, C, W);
+        } else {
+            todo &= ~(0xfu << lead);
+            px = lqx;
+            py = lqy;
+            pz = lqz;
+            active = true;
+            p.c0[0] = p.c1[0] = lx; p.c0[1] = p.c1[1] = ly; p.c0[2] = p.c1[2] = lz;
+            p.a[0] = p.b[0] = px; p.a[1] = p.b[1] = py; p.a[2] = p.b[2] = pz;
+            seed = __shfl_sync(0xffffffffu, seed, lead);
+            search<true>(m, active, px, py, pz, seed, p, cut2, g, C, W);
+        }
+        // what FP32 cannot tell apart from the nearest point, in FP64
+        float d1 = m.d1;
+        if (together) {
+            d1 = fminf(d1, __shfl_xor_sync(0xffffffffu, d1, 1));
+            d1 = fminf(d1, __shfl_xor_sync(0xffffffffu, d1, 2));
+        } else {
+            d1 = warp_min(d1);
+        }
+        const float limit = fmaf(d1, 3e-6f, d1) + 1e-36f;
+        double e = INFINITY;
+        bool again = active && !(d1 < INFINITY && d1 <= cut2 * 0.99997f);   // nothing within d_cut (cut2 carries a margin of 1e-5)
+        if (active && !again) {
+            if (m.d1 <= limit) e = dist2(px, py, pz, C.point[m.i1]);
+            if (m.d2 <= limit) e = fmin(e, dist2(px, py, pz, C.point[m.i2]));
+            again = m.d3 <= limit;
+        }
+        const unsigned crowd = __ballot_sync(0xffffffffu, again);
+        for (int o = 1; o < (together ? 4 : 32); o <<= 1) e = fmin(e, __shfl_xor_sync(0xffffffffu, e, o));
+        if (together) {
+            if (active && (lane & 3) == 0 && ((crowd >> lane) & 0xfu)) e = nn_exact(px, py, pz, p.k, g, C);
+            if (active) best = e;
+        } else if (lane == lead) {
+            best = crowd ? nn_exact(px, py, pz, p.k, g, C) : e;
+        }
+        __syncwarp();
+    }
+    if (mine && (lane & 3) == 0) d2[j] = best;
+}
+
+// step 2: distance, weight and integer weight of the squared distance, in place
+// of which the integer weight is stored.  FP64 throughout (some 80 operations
+// per candidate at 2 per clock and SM), so with full warps
+__global__ void k_mc_weight(long long n, double sigma, double eps, double *d, double *w, long long *wq) {
+    for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < n; j += (long long)gridDim.x * blockDim.x) {
+        const double best = __longlong_as_double(wq[j]);
         // nothing within the searched rings: the distance is at least d_cut, so the weight is eps
         const double wt = isinf(best) ? eps : fmax(exp(-best / (2.0 * sigma * sigma)), eps);
         if (d) d[j] = sqrt(best);
@@ -308,14 +823,30 @@ extern "C" MPM_API mpm_status mpm_mcis(int32_t n_obj, const int64_t *surf_off, c
     cudaStream_t st = (cudaStream_t)stream;
     const double cut = sigma * std::sqrt(2.0 * std::log(1.0 / eps));
     Grid g;
-    // cell edge 1/G >= d_cut / RINGS, so rings 0..RINGS hold every point within d_cut
+    // coarse cell edge 1/G >= d_cut / RINGS, so rings 0..RINGS hold every point within d_cut
     g.G = (int)std::floor(RINGS / cut);
     if (g.G < 1) g.G = 1;
     if (g.G > 256) g.G = 256;
+    if ((long long)g.G * g.G * g.G * n_obj >= (1ll << 31)) { g_mcis_msg = "mcis: grid too large"; return MPM_ERR_INVALID_ARG; }
+    // twice as fine where an object has the points to fill the cells (36,000
+    // points an object: 1.5 ms for 750k candidates, 2.1 ms with coarse cells,
+    // 1.7 ms four times as fine), while the mask stays within 8M words (its
+    // clearing and scan then cost some 30 us)
+    const int Gc = g.G;
+    auto mask_words = [&](int sub) {
+        const long long G = (long long)Gc * sub;
+        return n_obj * G * G * ((G + 31) / 32 + 1);
+    };
+    g.sub = ns / n_obj >= 2000 && mask_words(2) <= (1ll << 23) ? 2 : 1;
+    g.G = Gc * g.sub;
     g.inv_h = (float)g.G;
-    g.cells = (long long)g.G * g.G * g.G;
-    const long long keys = g.cells * n_obj;
-    if (keys >= (1ll << 31)) { g_mcis_msg = "mcis: grid too large"; return MPM_ERR_INVALID_ARG; }
+    g.zwords = (g.G + 31) / 32 + 1;
+    const long long words = mask_words(g.sub);
+    const float cut2 = (float)(cut * cut * (1.0 + 1e-5));
+    // the candidates' cells: up to twice the coarse grid's, about a warp's worth in one
+    int Gs = Gc;
+    if (8ll * Gc * Gc * Gc * n_obj <= (1ll << 23) && nc / n_obj >= 50000) Gs *= 2;
+    const long long keys = (long long)n_obj * Gs * Gs * Gs;
 
     // scratch: one stream-ordered allocation carved into pieces
     auto al = [](size_t b) { return (b + 255) & ~size_t(255); };
@@ -327,18 +858,29 @@ extern "C" MPM_API mpm_status mpm_mcis(int32_t n_obj, const int64_t *surf_off, c
     const size_t o_surf = off; off += al(ns * 12);
     const size_t o_cand = off; off += al(nc * 12);
     const size_t o_u = off; off += al(nd * 8);
-    const size_t o_cnt = off; off += al(keys * 4);
-    const size_t o_start = off; off += al(keys * 4);
-    const size_t o_rank = off; off += al(ns * 4);
+    // cleared together: mask, points per cell, boxes, candidates per cell
+    const size_t o_mask = off; off += al(words * 4);
+    const size_t o_cnt = off; off += al(ns * 4);
+    const size_t o_box = off; off += al(ns * 24);
     const size_t o_cnt2 = off; off += al(keys * 4);
+    const size_t o_clear = off;
+    const size_t o_bits = off; off += al(words * 4);
+    const size_t o_before = off; off += al(words * 4);
+    const size_t o_start = off; off += al(ns * 4);
+    const size_t o_cell = off; off += al(ns * 4);
+    const size_t o_rank = off; off += al(ns * 4);
+    const size_t o_lo = off; off += al(ns * 16);
+    const size_t o_hi = off; off += al(ns * 16);
     const size_t o_start2 = off; off += al(keys * 4);
+    const size_t o_ccell = off; off += al(nc * 4);
     const size_t o_crank = off; off += al(nc * 4);
     const size_t o_order = off; off += al(nc * 4);
     const size_t o_sorted = off; off += al(ns * 16);
     const size_t o_wq = off; off += al(nc * 8);
     const size_t o_cum = off; off += al(nc * 8);
     const size_t o_tot = off; off += al((nb + 1) * 8);
-    const size_t o_kb = off; off += al(((keys + SC_T - 1) / SC_T + 1) * 8);   // cell-count scan block sums
+    const long long scan_most = std::max(keys, std::max(words, ns));
+    const size_t o_kb = off; off += al(((scan_most + SC_T - 1) / SC_T + 1) * 8);   // scan block sums
     const size_t o_kt = off; off += al(8);
     const size_t o_d = off; off += al(nc * 8);
     const size_t o_w = off; off += al(nc * 8);
@@ -369,33 +911,39 @@ extern "C" MPM_API mpm_status mpm_mcis(int32_t n_obj, const int64_t *surf_off, c
         if (ns > 0 && !is_dev(surf)) { MC_CK(cudaMemcpyAsync(P(o_surf), surf, ns * 12, cudaMemcpyHostToDevice, st)); dsurf = (const float *)P(o_surf); }
         if (nc > 0 && !is_dev(cand)) { MC_CK(cudaMemcpyAsync(P(o_cand), cand, nc * 12, cudaMemcpyHostToDevice, st)); dcand = (const float *)P(o_cand); }
         if (nd > 0 && !is_dev(u)) { MC_CK(cudaMemcpyAsync(P(o_u), u, nd * 8, cudaMemcpyHostToDevice, st)); du = (const double *)P(o_u); }
-        unsigned *cnt = (unsigned *)P(o_cnt), *start = (unsigned *)P(o_start), *rank = (unsigned *)P(o_rank);
-        unsigned *cnt2 = (unsigned *)P(o_cnt2), *start2 = (unsigned *)P(o_start2);
-        float4 *sorted = (float4 *)P(o_sorted);
+        auto U = [&](size_t o) { return (unsigned *)P(o); };
+        unsigned *mask = U(o_mask), *cnt = U(o_cnt), *start = U(o_start);
+        unsigned long long *kb = (unsigned long long *)P(o_kb), *kt = (unsigned long long *)P(o_kt);
+        const Cells cells = {mask, U(o_before), (const float4 *)P(o_lo), (const float4 *)P(o_hi), (const float4 *)P(o_sorted)};
         long long *wq = (long long *)P(o_wq), *cum = (long long *)P(o_cum), *tot = (long long *)P(o_tot);
-        MC_CK(cudaMemsetAsync(cnt, 0, keys * 4, st));
+        MC_CK(cudaMemsetAsync(mask, 0, o_clear - o_mask, st));
         if (ns > 0) {
-            k_mc_count<<<blocks_for(ns, 256), 256, 0, st>>>(n_obj, dsoff, dsurf, g, cnt, rank);
-            MC_CK(cudaGetLastError());
-        }
-        scan_counts(cnt, start, keys, (unsigned long long *)P(o_kb), (unsigned long long *)P(o_kt), st);
-        MC_CK(cudaGetLastError());
-        if (ns > 0) {
-            k_mc_scatter<<<blocks_for(ns, 256), 256, 0, st>>>(n_obj, dsoff, dsurf, g, start, rank, sorted);
+            k_mc_mark<<<blocks_for(ns, 256), 256, 0, st>>>(n_obj, dsoff, dsurf, g, mask);
+            k_mc_bits<<<blocks_for(words, 256), 256, 0, st>>>(mask, words, U(o_bits));
+            scan_counts(U(o_bits), U(o_before), words, kb, kt, st);
+            k_mc_count<<<blocks_for(ns, 256), 256, 0, st>>>(n_obj, dsoff, dsurf, g, mask, U(o_before), cnt, U(o_cell),
+                                                            U(o_rank), U(o_box));
+            scan_counts(cnt, start, ns, kb, kt, st);
+            k_mc_scatter<<<blocks_for(ns, 256), 256, 0, st>>>(ns, dsurf, start, U(o_cell), U(o_rank), cnt, U(o_box),
+                                                              (float4 *)P(o_sorted), (float4 *)P(o_lo),
+                                                              (float4 *)P(o_hi));
             MC_CK(cudaGetLastError());
         }
         double *dd = d && is_dev(d) ? d : (double *)P(o_d);
         double *dw = w && is_dev(w) ? w : (double *)P(o_w);
         int64_t *dp = picked && is_dev(picked) ? picked : (int64_t *)P(o_pick);
         if (nc > 0) {
-            unsigned *crank = (unsigned *)P(o_crank), *order = (unsigned *)P(o_order);
-            MC_CK(cudaMemsetAsync(cnt2, 0, keys * 4, st));
-            k_mc_cand_count<<<blocks_for(nc, 256), 256, 0, st>>>(n_obj, dcoff, dcand, g, cnt2, crank);
-            scan_counts(cnt2, start2, keys, (unsigned long long *)P(o_kb), (unsigned long long *)P(o_kt), st);
-            k_mc_cand_scatter<<<blocks_for(nc, 256), 256, 0, st>>>(n_obj, dcoff, dcand, g, start2, crank, order);
+            unsigned *cnt2 = U(o_cnt2), *start2 = U(o_start2), *order = U(o_order);
+            k_mc_cand_count<<<blocks_for(nc, 256), 256, 0, st>>>(n_obj, dcoff, dcand, Gs, cnt2, U(o_ccell), U(o_crank));
+            scan_counts(cnt2, start2, keys, kb, kt, st);
+            k_mc_cand_scatter<<<blocks_for(nc, 256), 256, 0, st>>>(nc, start2, U(o_ccell), U(o_crank), order);
             MC_CK(cudaGetLastError());
-            k_mc_nn<<<blocks_for(nc, 128), 128, 0, st>>>(n_obj, dcoff, dcand, order, g, start, cnt, sorted, sigma, eps,
-                                                           dd, dw, wq);
+            // candidates per warp: 8, fewer where that would leave SMs without warps
+            const int per = (int)std::min<long long>(TURN, std::max<long long>(1, nc / (152 * 24)));
+            const long long ctas = (nc + per * NN_WARPS - 1) / (per * NN_WARPS);
+            k_mc_nn<<<(unsigned)ctas, 32 * NN_WARPS, 0, st>>>(n_obj, dsoff, dcoff, dcand, order, g, cells, per,
+                                                              std::max(1, g.sub / 2), (float)Gs, cut2, (double *)wq);
+            k_mc_weight<<<blocks_for(nc, 256), 256, 0, st>>>(nc, sigma, eps, dd, dw, wq);
             MC_CK(cudaGetLastError());
             k_mc_scan_i64_block<<<(unsigned)nb, 1024, 0, st>>>(wq, cum, nc, tot);
             k_mc_scan_i64_totals<<<1, 1024, 0, st>>>(tot, nb);
