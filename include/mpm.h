@@ -28,6 +28,10 @@
  *  - stream: a cudaStream_t, or NULL for the legacy default stream.  Calls
  *    enqueue work on it; they do not synchronise unless stated.
  *
+ *  - mpm_mcis and mpm_render, which have no context, take their scratch from a
+ *    memory pool of the library's that keeps up to 256 MiB per device between
+ *    calls; destroying the last context gives it back.
+ *
  * Errors
  *  - Every entry point returns mpm_status; no C++ exception crosses the ABI.
  *  - Argument checks are synchronous.  Conditions found on the device

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstdint>
@@ -15,6 +16,7 @@
 
 #include "../../include/mpm.h"
 #include "mpm_internal.h"
+#include "mpm_scratch.h"
 
 using namespace mpm;
 
@@ -22,6 +24,7 @@ namespace {
 
 const char *g_create_error = "";
 thread_local std::string g_create_msg;
+std::atomic<int> g_contexts{0};   // contexts alive
 
 }  // namespace
 
@@ -512,6 +515,7 @@ MPM_API mpm_status mpm_create(const int32_t grid_res[3], float dx, float dt, con
 
     mpm_ctx *ctx = new (std::nothrow) mpm_ctx();
     if (!ctx) { g_create_error = "host allocation failed"; return MPM_ERR_OOM; }
+    ++g_contexts;
     cudaGetDevice(&ctx->device);
     cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, ctx->device);
     std::memset(&ctx->D, 0, sizeof(Dev));
@@ -787,6 +791,7 @@ MPM_API mpm_status mpm_destroy(mpm_ctx *ctx) {
         if (g) cudaGraphExecDestroy(g);
     if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
     delete ctx;
+    if (--g_contexts == 0) scratch_trim();
     return MPM_OK;
 }
 

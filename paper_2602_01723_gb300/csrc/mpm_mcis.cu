@@ -32,6 +32,7 @@
 #include "../../include/mpm.h"
 #include "mpm_ptr.h"
 #include "mpm_scan.cuh"
+#include "mpm_scratch.h"
 
 namespace {
 
@@ -886,7 +887,7 @@ extern "C" MPM_API mpm_status mpm_mcis(int32_t n_obj, const int64_t *surf_off, c
     const size_t o_w = off; off += al(nc * 8);
     const size_t o_pick = off; off += al(nd * 8);
     char *buf = nullptr;
-    if (cudaMallocAsync((void **)&buf, off ? off : 256, st) != cudaSuccess) {
+    if (mpm::scratch_alloc((void **)&buf, off ? off : 256, st) != cudaSuccess) {
         cudaGetLastError();
         g_mcis_msg = "mcis: device allocation failed";
         return MPM_ERR_OOM;

@@ -26,6 +26,7 @@
 #include "../../include/mpm.h"
 #include "mpm_ptr.h"
 #include "mpm_scan.cuh"
+#include "mpm_scratch.h"
 
 namespace {
 
@@ -287,7 +288,7 @@ extern "C" MPM_API mpm_status mpm_render(int64_t n, const float *mean, const flo
         const size_t o_rng = off; off += al(tiles * 8);
         const size_t o_img = off; off += al(npix * 12);
         const size_t o_tr = off; off += al(npix * 4);
-        if (cudaMallocAsync((void **)&buf, off, st) != cudaSuccess) {
+        if (mpm::scratch_alloc((void **)&buf, off, st) != cudaSuccess) {
             cudaGetLastError();
             buf = nullptr;
             g_render_msg = "render: device allocation failed";
@@ -326,7 +327,7 @@ extern "C" MPM_API mpm_status mpm_render(int64_t n, const float *mean, const flo
             const size_t o_ho = ko; ko += al((size_t)256 * nb * 4);
             const size_t o_ht = ko; ko += al(8);
             const size_t o_hb = ko; ko += al(((256ll * nb + SC_T - 1) / SC_T + 1) * 8);
-            if (cudaMallocAsync((void **)&kbuf, ko, st) != cudaSuccess) {
+            if (mpm::scratch_alloc((void **)&kbuf, ko, st) != cudaSuccess) {
                 cudaGetLastError();
                 kbuf = nullptr;
                 g_render_msg = "render: device allocation failed";
