@@ -859,7 +859,8 @@ extern "C" MPM_API mpm_status mpm_mcis(int32_t n_obj, const int64_t *surf_off, c
     const size_t o_surf = off; off += al(ns * 12);
     const size_t o_cand = off; off += al(nc * 12);
     const size_t o_u = off; off += al(nd * 8);
-    // cleared together: mask, points per cell, boxes, candidates per cell
+    // cleared together: the scans' ticket, mask, points per cell, boxes, candidates per cell
+    const size_t o_ticket = off; off += al(4);
     const size_t o_mask = off; off += al(words * 4);
     const size_t o_cnt = off; off += al(ns * 4);
     const size_t o_box = off; off += al(ns * 24);
@@ -881,7 +882,7 @@ extern "C" MPM_API mpm_status mpm_mcis(int32_t n_obj, const int64_t *surf_off, c
     const size_t o_cum = off; off += al(nc * 8);
     const size_t o_tot = off; off += al((nb + 1) * 8);
     const long long scan_most = std::max(keys, std::max(words, ns));
-    const size_t o_kb = off; off += al(((scan_most + SC_T - 1) / SC_T + 1) * 8);   // scan block sums
+    const size_t o_kb = off; off += al(scan_words(scan_most) * 8);   // scan block sums
     const size_t o_kt = off; off += al(8);
     const size_t o_d = off; off += al(nc * 8);
     const size_t o_w = off; off += al(nc * 8);
@@ -917,14 +918,15 @@ extern "C" MPM_API mpm_status mpm_mcis(int32_t n_obj, const int64_t *surf_off, c
         unsigned long long *kb = (unsigned long long *)P(o_kb), *kt = (unsigned long long *)P(o_kt);
         const Cells cells = {mask, U(o_before), (const float4 *)P(o_lo), (const float4 *)P(o_hi), (const float4 *)P(o_sorted)};
         long long *wq = (long long *)P(o_wq), *cum = (long long *)P(o_cum), *tot = (long long *)P(o_tot);
-        MC_CK(cudaMemsetAsync(mask, 0, o_clear - o_mask, st));
+        unsigned *ticket = U(o_ticket);
+        MC_CK(cudaMemsetAsync(ticket, 0, o_clear - o_ticket, st));
         if (ns > 0) {
             k_mc_mark<<<blocks_for(ns, 256), 256, 0, st>>>(n_obj, dsoff, dsurf, g, mask);
             k_mc_bits<<<blocks_for(words, 256), 256, 0, st>>>(mask, words, U(o_bits));
-            scan_counts(U(o_bits), U(o_before), words, kb, kt, st);
+            scan_counts(U(o_bits), U(o_before), words, kb, kt, ticket, st);
             k_mc_count<<<blocks_for(ns, 256), 256, 0, st>>>(n_obj, dsoff, dsurf, g, mask, U(o_before), cnt, U(o_cell),
                                                             U(o_rank), U(o_box));
-            scan_counts(cnt, start, ns, kb, kt, st);
+            scan_counts(cnt, start, ns, kb, kt, ticket, st);
             k_mc_scatter<<<blocks_for(ns, 256), 256, 0, st>>>(ns, dsurf, start, U(o_cell), U(o_rank), cnt, U(o_box),
                                                               (float4 *)P(o_sorted), (float4 *)P(o_lo),
                                                               (float4 *)P(o_hi));
@@ -936,7 +938,7 @@ extern "C" MPM_API mpm_status mpm_mcis(int32_t n_obj, const int64_t *surf_off, c
         if (nc > 0) {
             unsigned *cnt2 = U(o_cnt2), *start2 = U(o_start2), *order = U(o_order);
             k_mc_cand_count<<<blocks_for(nc, 256), 256, 0, st>>>(n_obj, dcoff, dcand, Gs, cnt2, U(o_ccell), U(o_crank));
-            scan_counts(cnt2, start2, keys, kb, kt, st);
+            scan_counts(cnt2, start2, keys, kb, kt, ticket, st);
             k_mc_cand_scatter<<<blocks_for(nc, 256), 256, 0, st>>>(nc, start2, U(o_ccell), U(o_crank), order);
             MC_CK(cudaGetLastError());
             // candidates per warp: 8, fewer where that would leave SMs without warps

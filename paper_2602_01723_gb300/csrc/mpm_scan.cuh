@@ -5,12 +5,14 @@
 
 namespace {
 
-// exclusive scan of n unsigned counts over many CTAs, three phases:
-//   1. each CTA scans its 1024 counts and stores their sum in btot[block];
-//   2. one CTA scans the block sums (exclusive, in place) and writes the
-//      grand total to *total;
-//   3. each CTA adds its block's offset.
-constexpr int SC_T = 1024;
+// Exclusive scan of n unsigned counts over many CTAs.  Each CTA scans its SC_N
+// counts and stores their sum; the last CTA to finish scans the sums (exclusive,
+// in place) and writes the grand total, so that the scan is one launch.  A CTA's
+// offset, its scanned sum, is added by a second launch (scan_counts) or by the
+// kernel that reads the scan (scan_blocks, scanned).
+constexpr int SC_T = 1024;            // threads per CTA
+constexpr int SC_V = 4;               // consecutive counts per thread
+constexpr int SC_N = SC_T * SC_V;
 __device__ __forceinline__ unsigned long long block_exclusive_scan(unsigned long long v, unsigned long long &tot) {
     __shared__ unsigned long long sh[SC_T / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -35,38 +37,69 @@ __device__ __forceinline__ unsigned long long block_exclusive_scan(unsigned long
     __syncthreads();
     return ex;
 }
-__global__ void __launch_bounds__(SC_T) k_sc_block(const unsigned *in, unsigned *out, long long n,
-                                                   unsigned long long *btot) {
-    const long long i = blockIdx.x * (long long)SC_T + threadIdx.x;
-    unsigned long long tot;
-    const unsigned long long ex = block_exclusive_scan(i < n ? in[i] : 0u, tot);
-    if (i < n) out[i] = (unsigned)ex;
-    if (threadIdx.x == 0) btot[blockIdx.x] = tot;
-}
-__global__ void __launch_bounds__(SC_T) k_sc_totals(unsigned long long *btot, long long nb, unsigned long long *total) {
-    unsigned long long carry = 0;
-    for (long long b0 = 0; b0 < nb; b0 += SC_T) {
-        const long long i = b0 + threadIdx.x;
-        unsigned long long tot;
-        const unsigned long long ex = block_exclusive_scan(i < nb ? btot[i] : 0ull, tot);
-        if (i < nb) btot[i] = carry + ex;
-        carry += tot;
+// order (nullable): count i is in[order[i]].  ticket: zero before the launch, and after it.
+__global__ void __launch_bounds__(SC_T) k_sc_block(const unsigned *in, const unsigned *order, unsigned *out, long long n,
+                                                   unsigned long long *btot, unsigned long long *total,
+                                                   unsigned *ticket) {
+    const long long i0 = blockIdx.x * (long long)SC_N + threadIdx.x * SC_V;
+    unsigned v[SC_V];
+    unsigned long long sum = 0;
+#pragma unroll
+    for (int u = 0; u < SC_V; ++u) {
+        v[u] = i0 + u < n ? in[order ? order[i0 + u] : i0 + u] : 0u;
+        sum += v[u];
     }
-    if (threadIdx.x == 0) *total = carry;
+    unsigned long long tot;
+    unsigned long long ex = block_exclusive_scan(sum, tot);
+#pragma unroll
+    for (int u = 0; u < SC_V; ++u) {
+        if (i0 + u < n) out[i0 + u] = (unsigned)ex;
+        ex += v[u];
+    }
+    __shared__ bool last;
+    if (threadIdx.x == 0) {
+        btot[blockIdx.x] = tot;
+        __threadfence();
+        last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    unsigned long long carry = 0;
+    for (long long b0 = 0; b0 < gridDim.x; b0 += SC_T) {
+        const long long i = b0 + threadIdx.x;
+        const unsigned long long x = i < gridDim.x ? __ldcg(&btot[i]) : 0ull;
+        unsigned long long t;
+        const unsigned long long e = block_exclusive_scan(x, t);
+        if (i < gridDim.x) btot[i] = carry + e;
+        carry += t;
+    }
+    if (threadIdx.x == 0) {
+        *total = carry;
+        *ticket = 0;
+    }
 }
 __global__ void __launch_bounds__(SC_T) k_sc_add(unsigned *out, long long n, const unsigned long long *btot) {
-    const long long i = blockIdx.x * (long long)SC_T + threadIdx.x;
-    if (i < n) out[i] += (unsigned)btot[blockIdx.x];
+    for (long long i = blockIdx.x * (long long)SC_N + threadIdx.x; i < min(n, (blockIdx.x + 1) * (long long)SC_N); i += SC_T)
+        out[i] += (unsigned)btot[blockIdx.x];
 }
 
-// exclusive scan of n counts into out (sums below 2^32), grand total to *total;
-// btot: ceil(n / SC_T) scratch words
-inline void scan_counts(const unsigned *in, unsigned *out, long long n, unsigned long long *btot, unsigned long long *total,
-                 cudaStream_t st) {
-    const long long nb = (n + SC_T - 1) / SC_T;
-    if (nb > 0) k_sc_block<<<(unsigned)nb, SC_T, 0, st>>>(in, out, n, btot);
-    k_sc_totals<<<1, SC_T, 0, st>>>(btot, nb, total);
-    if (nb > 0) k_sc_add<<<(unsigned)nb, SC_T, 0, st>>>(out, n, btot);
+// 64-bit scratch words for the block sums of a scan of up to n counts
+inline long long scan_words(long long n) { return (n + SC_N - 1) / SC_N + 1; }
+// the scan without the CTAs' offsets: count i's prefix is out[i] + btot[i / SC_N] (scanned)
+inline void scan_blocks(const unsigned *in, const unsigned *order, unsigned *out, long long n, unsigned long long *btot,
+                        unsigned long long *total, unsigned *ticket, cudaStream_t st) {
+    if (n > 0) k_sc_block<<<(unsigned)((n + SC_N - 1) / SC_N), SC_T, 0, st>>>(in, order, out, n, btot, total, ticket);
+}
+__device__ __forceinline__ unsigned scanned(const unsigned *out, const unsigned long long *btot, long long i) {
+    return out[i] + (unsigned)btot[i / SC_N];
+}
+// exclusive scan of n counts into out (sums below 2^32), grand total to *total
+// (unchanged for n = 0); btot: scan_words(n) scratch words; ticket: one zero word, left zero
+inline void scan_counts(const unsigned *in, unsigned *out, long long n, unsigned long long *btot,
+                        unsigned long long *total, unsigned *ticket, cudaStream_t st) {
+    scan_blocks(in, nullptr, out, n, btot, total, ticket, st);
+    if (n > SC_N) k_sc_add<<<(unsigned)((n + SC_N - 1) / SC_N), SC_T, 0, st>>>(out, n, btot);
 }
 
 }  // namespace
