@@ -313,7 +313,7 @@ static void middle_direct(mpm_ctx *ctx, int s, cudaStream_t st, bool keep) {
 // with the ordered one).  A launch of a graph costs about 3 us of idle GPU:
 // the longer one takes the 8k cube from 14.0 to 12.3 us per substep and the
 // 300k scene from 57.0 to 55.0, and is worth its instantiation in a first run
-// of 100 substeps.  It is captured on a library-owned stream (the legacy
+// of more than two periods; a shorter first run does with the pair.  It is captured on a library-owned stream (the legacy
 // default stream cannot be captured) the first time it is needed for this
 // particle count and these buffers, and replayed on the caller's stream.
 static cudaGraphExec_t steady_graph(mpm_ctx *ctx, cudaStream_t st, bool direct, int len) {
@@ -399,7 +399,7 @@ mpm_status run_substeps(mpm_ctx *ctx, int n_sub, cudaStream_t st, float4 *tape, 
         };
         for (int s = 1; s < middle;) {
             int len = 0;
-            if (s % REORDER == 1) len = replay(s, REORDER) * REORDER;
+            if (s % REORDER == 1 && (ctx->ran_direct || middle > 2 * REORDER)) len = replay(s, REORDER) * REORDER;
             if (!len && (s & 1) && (s + 1) % REORDER) len = replay(s, 2) * 2;
             if (len < 0) return fail(ctx, MPM_ERR_CUDA, "graph launch failed");
             if (!len) {
@@ -412,6 +412,7 @@ mpm_status run_substeps(mpm_ctx *ctx, int n_sub, cudaStream_t st, float4 *tape, 
         L_between(ctx, middle & 1, -1, st);              // work items of the last binning
         L_substep(ctx, 2, middle & 1, 0, st, false, middle & 1);
         ctx->bins_pending = true;     // the last substep binned the new positions (for a sort)
+        ctx->ran_direct = true;
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return fail(ctx, MPM_ERR_CUDA, std::string("launch: ") + cudaGetErrorString(e));
         return MPM_OK;
@@ -646,9 +647,9 @@ MPM_API mpm_status mpm_load_particles(mpm_ctx *ctx, int64_t n, const float *x, c
     CK(cudaMemsetAsync(D.bcount, 0, (size_t)ctx->total_blocks * sizeof(unsigned), st));
     CK(cudaMemsetAsync(D.ctr + CTR_N_OCC, 0, sizeof(unsigned), st));
     CK(cudaMemsetAsync(D.ctr + CTR_D_OVF_TOTAL, 0, 2 * sizeof(unsigned), st));   // and CTR_MAX_COUNT
-    launch_load(D, a, st);
+    launch_load(D, a, st);   // and the binning of the positions
     ++ctx->launches;
-    L_bin(ctx, st);
+    ctx->bins_pending = true;
     CKLAUNCH();
     ctx->sticky = MPM_OK;
     ctx->loaded = true;

@@ -44,7 +44,7 @@ inline int grid_for(long long n, int threads, int cap = 152 * 16) {
     return (int)g;
 }
 
-void launch_load(const Dev &D, const LoadArgs &a, cudaStream_t st);
+void launch_load(const Dev &D, const LoadArgs &a, cudaStream_t st);   // bins the particles too
 void launch_bin(const Dev &D, cudaStream_t st);
 void launch_plan(const Dev &D, int bump_mask, cudaStream_t st);
 void launch_prepare(const Dev &D, int upd_par, int act_par, int do_sort, int keep_momentum, int grid, cudaStream_t st);
@@ -156,6 +156,7 @@ struct mpm_ctx {
     // CUDA graphs of steady-state substeps: [0] two (one per grid-buffer
     // parity), [1] a whole reordering period of a direct-binning run
     bool use_graph = true;
+    bool ran_direct = false;             // a direct-binning run has been made
     cudaStream_t cap_stream = nullptr;   // library-owned stream the graphs are captured on
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
     long long graph_key[2] = {-1, -1};   // (n, buffer generation, binning) each was captured for
