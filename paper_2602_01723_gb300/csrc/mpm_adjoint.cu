@@ -357,28 +357,7 @@ constexpr int ADJ_THREADS = 128;
 //   ADJ_FCR_NH   fixed-corotated and Neo-Hookean
 //   ADJ_ALL      also StVK, Hencky, fluid and volume elasticity
 
-__device__ __forceinline__ int page_slot_a(const Dev &D, int par, unsigned ep, int inst, int bx, int by, int bz) {
-    if (bx < 0 || by < 0 || bz < 0 || bx >= D.NB[0] || by >= D.NB[1] || bz >= D.NB[2]) return -1;
-    const unsigned k = block_key(D, inst, bx, by, bz);
-    return D.page_epoch[par][k] == ep ? D.page[par][k] : -1;
-}
 __device__ __forceinline__ int node_loc(int I, int J, int K) { return ((I & 3) * 4 + (J & 3)) * 4 + (K & 3); }
-
-// loads the 6^3-node tile (blocks B .. B+1) of pool `src` into shared memory
-__device__ void load_tile(const Dev &D, const float4 *src, unsigned ep, int inst, int bx, int by, int bz,
-                          float4 *tile, int *slots) {
-    if (threadIdx.x < 8) {
-        const int o = threadIdx.x;
-        slots[o] = page_slot_a(D, 0, ep, inst, bx + (o >> 2), by + ((o >> 1) & 1), bz + (o & 1));
-    }
-    __syncthreads();
-    for (int t = threadIdx.x; t < GT3; t += blockDim.x) {
-        const int i = t / (GT * GT), j = (t / GT) % GT, k = t % GT;
-        const int sl = slots[((i >> 2) << 2) | ((j >> 2) << 1) | (k >> 2)];
-        tile[t] = sl >= 0 ? src[(size_t)sl * BLK_NODES + node_loc(i, j, k)] : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    __syncthreads();
-}
 
 struct ParticleIn {
     int q[3];                      // fixed-point position (cells = q 2^-qf)
@@ -400,28 +379,36 @@ __device__ __forceinline__ void unpack_particle(const float4 r[REC_F4], Particle
     P.alpha = r[7].w;
 }
 
+// Strides of the 6^3-node tiles, in nodes: 1, 8, 52.  The 64 base cells of a
+// block then cover the 32 banks of a plane of words exactly twice each, and the
+// 8 groups of 16 bytes of a float4 tile evenly: lanes whose cells differ in
+// that order, as the forward's lists have them, read and add without conflicts.
+constexpr int GTI = GT * 8 + 4;
+constexpr int GTN = GT * GTI;                // nodes of a tile, with the gaps
+constexpr int GT3P = GTN + 8;                // 320 = 10 x 32: every component starts at bank 0
+__device__ __forceinline__ int gidx(int i, int j, int k) { return i * GTI + j * 8 + k; }
+
 // shared memory of the reverse G2P kernel
-constexpr int GTP = GT + 1;                  // padded row of the fixed-point tile
-constexpr int GT3P = GT * GT * GTP;
-__device__ __forceinline__ int gidx(int i, int j, int k) { return (i * GT + j) * GTP + k; }
 constexpr int AS_F4 = 13;                   // staged stride: record words 0,1,4..7 (6) + adjoint (6), odd
 struct AdjG2PSmem {
     float4 st[ADJ_THREADS * AS_F4];          // staged record and adjoint of the chunk's particles
-    float4 g[GT3];                           // grid velocity tile (v, m)
+    float2 gxy[GTN];                         // grid velocity tile: v0, v1 per node
+    float gz[GTN];                           // ... and v2
     int t[3 * GT3P];                         // fixed-point grid-velocity adjoint, component-major
-    float4 pk[ADJ_THREADS * 4];              // packets: f(3) - | vt(3) - | Ct(9) ...
     int4 cd[3];                              // chunk descriptors, ring of (c, c + G, c + 2G)
     unsigned pidx[ADJ_THREADS];              // sorted indices of the next chunk
     unsigned pe[8];                          // page words of the next chunk's 8 tile blocks
     int ps[8];
     int slot[2][8];                          // pool slots of the tile blocks, per chunk parity
     float red[ADJ_THREADS / 32];
-    float scale;
 };
 
 __device__ __forceinline__ unsigned a_smem(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void a_cp16(void *dst, const void *src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"(a_smem(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void a_cp8(void *dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(a_smem(dst)), "l"(src) : "memory");
 }
 __device__ __forceinline__ void a_cp4(void *dst, const void *src) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(a_smem(dst)), "l"(src) : "memory");
@@ -447,14 +434,14 @@ __device__ __forceinline__ void adj_stage2(const Dev &D, SM &S, int4 ch, unsigne
     if (tid < ch.z) a_cp4(&S.pidx[tid], D.sorted + ch.y + tid);
     const int t = tid - 64;   // lookups on the third warp
     if (t >= 0 && t < 8) {
-        int inst, bx, by, bz;
-        key_coords(D, (unsigned)ch.x, inst, bx, by, bz);
+        int bx, by, bz;
+        item_coords(ch.w, bx, by, bz);
         const int qx = bx + (t >> 2), qy = by + ((t >> 1) & 1), qz = bz + (t & 1);
         if (qx >= D.NB[0] || qy >= D.NB[1] || qz >= D.NB[2]) {
             S.pe[t] = ep + 1u;
             S.ps[t] = -1;
         } else {
-            const unsigned k = block_key(D, inst, qx, qy, qz);
+            const unsigned k = key_offset(D, (unsigned)ch.x, qx - bx, qy - by, qz - bz);
             a_cp4(&S.pe[t], D.page_epoch[0] + k);
             a_cp4(&S.ps[t], D.page[0] + k);
         }
@@ -480,8 +467,15 @@ __device__ __forceinline__ void adj_stage3(const Dev &D, AdjG2PSmem &S, int4 ch,
         const int i = t / (GT * GT), j = (t / GT) % GT, k = t % GT;
         const int b = ((i >> 2) << 2) | ((j >> 2) << 1) | (k >> 2);
         const int sl = S.pe[b] == ep ? S.ps[b] : -1;
-        if (sl >= 0) a_cp16(&S.g[t], D.gv[0] + (size_t)sl * BLK_NODES + node_loc(i, j, k));
-        else S.g[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+        const int q = gidx(i, j, k);
+        if (sl >= 0) {
+            const float4 *src = D.gv[0] + (size_t)sl * BLK_NODES + node_loc(i, j, k);
+            a_cp8(&S.gxy[q], src);
+            a_cp4(&S.gz[q], &src->z);
+        } else {
+            S.gxy[q] = make_float2(0.f, 0.f);
+            S.gz[q] = 0.f;
+        }
     }
 }
 
@@ -535,8 +529,8 @@ __global__ void __launch_bounds__(ADJ_THREADS, 3) k_adj_g2p(Dev D, const float4 
         if (tid == 0 && cn + gridDim.x < n_chunks) a_cp16(&S.cd[(kc + 2) % 3], D.chunks + cn + gridDim.x);
         if (has_next) adj_stage2(D, S, S.cd[(kc + 1) % 3], ep);
         a_commit();
-        int inst, bx, by, bz;
-        key_coords(D, (unsigned)ch.x, inst, bx, by, bz);
+        int bx, by, bz;
+        item_coords(ch.w, bx, by, bz);
         float4 rr[REC_F4], aa[ADJ_F4];
         if (valid) {
             const float4 *q = S.st + tid * AS_F4;
@@ -545,12 +539,14 @@ __global__ void __launch_bounds__(ADJ_THREADS, 3) k_adj_g2p(Dev D, const float4 
             for (int w = 0; w < ADJ_F4; ++w) aa[w] = q[6 + w];
         }
         float bnd = 0.f;
+        // what the particle scatters to the grid-velocity adjoint, kept in
+        // registers: cell and offset in the tile, velocity and affine adjoints
+        float f[3], vt[3], Ct[9];
+        int b[3];
         if (valid) {
             rr[2] = rr[3] = make_float4(0.f, 0.f, 0.f, 0.f);
             ParticleIn P;
             unpack_particle(rr, P);
-            float f[3];
-            int b[3];
             b[0] = base_cell_q(P.q[0], D, f[0]) - bx * BLK;
             b[1] = base_cell_q(P.q[1], D, f[1]) - by * BLK;
             b[2] = base_cell_q(P.q[2], D, f[2]) - bz * BLK;
@@ -566,7 +562,8 @@ __global__ void __launch_bounds__(ADJ_THREADS, 3) k_adj_g2p(Dev D, const float4 
             const float Fb[9] = {aa[3].w, aa[4].x, aa[4].y, aa[4].z, aa[4].w, aa[5].x, aa[5].y, aa[5].z, aa[5].w};
             // x' = x + dt v': the velocity's total adjoint
             float xa[3] = {xb[0], xb[1], xb[2]};
-            const float vt[3] = {vb[0] + dt * xb[0], vb[1] + dt * xb[1], vb[2] + dt * xb[2]};
+#pragma unroll
+            for (int t = 0; t < 3; ++t) vt[t] = vb[t] + dt * xb[t];
             // The reverse of the gathers v' = sum w v_i and C' = c4 sum w v_i (x_i - x_p)^T
             // gives the position adjoint sum_i wbar_i grad w_i - c4 Ct^T sum_i w_i v_i,
             // with wbar_i = vt . v_i + c4 v_i^T Ct (x_i - x_p) and Ct the total adjoint
@@ -575,7 +572,6 @@ __global__ void __launch_bounds__(ADJ_THREADS, 3) k_adj_g2p(Dev D, const float4 
             // on C', so one pass over the 27 nodes recomputes v', C' and accumulates
             // the first term; with plasticity Ct needs the return map of C', and a
             // second pass follows.
-            float Ct[9];
             float vn[3] = {0.f, 0.f, 0.f}, Bm[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
             if (MS == ADJ_ELASTIC) {
 #pragma unroll
@@ -594,7 +590,9 @@ __global__ void __launch_bounds__(ADJ_THREADS, 3) k_adj_g2p(Dev D, const float4 
                     for (int k = 0; k < 3; ++k) {
                         const float wij = w[0][i] * w[1][jj];
                         const float wt = wij * w[2][k];
-                        const float4 g = S.g[((b[0] + i) * GT + (b[1] + jj)) * GT + (b[2] + k)];
+                        const int nd = gidx(b[0] + i, b[1] + jj, b[2] + k);
+                        const float2 gxy = S.gxy[nd];
+                        const float3 g = make_float3(gxy.x, gxy.y, S.gz[nd]);
                         const float dd[3] = {(float)i - f[0], (float)jj - f[1], (float)k - f[2]};
                         const float a3[3] = {wt * g.x, wt * g.y, wt * g.z};
 #pragma unroll
@@ -659,12 +657,13 @@ __global__ void __launch_bounds__(ADJ_THREADS, 3) k_adj_g2p(Dev D, const float4 
                     const float wi = i == 0 ? w[0][0] : (i == 1 ? w[0][1] : w[0][2]);
                     const float dwi = i == 0 ? dw[0][0] : (i == 1 ? dw[0][1] : dw[0][2]);
                     const float di = (float)i - f[0];
-                    const float4 *gi = S.g + (b[0] + i) * GT * GT;
+                    const int ndi = gidx(b[0] + i, b[1], b[2]);
 #pragma unroll
                     for (int jj = 0; jj < 3; ++jj)
 #pragma unroll
                         for (int k = 0; k < 3; ++k) {
-                            const float4 g = gi[(b[1] + jj) * GT + (b[2] + k)];
+                            const float2 gxy = S.gxy[ndi + jj * 8 + k];
+                            const float3 g = make_float3(gxy.x, gxy.y, S.gz[ndi + jj * 8 + k]);
                             const float dd[3] = {di, (float)jj - f[1], (float)k - f[2]};
                             const float vi[3] = {g.x, g.y, g.z};
                             float wbar = 0.f;
@@ -681,30 +680,23 @@ __global__ void __launch_bounds__(ADJ_THREADS, 3) k_adj_g2p(Dev D, const float4 
             // - c4 Ct^T v'
 #pragma unroll
             for (int cc = 0; cc < 3; ++cc) xa[cc] -= c4 * (Ct[cc] * vn[0] + Ct[3 + cc] * vn[1] + Ct[6 + cc] * vn[2]);
+            // the reverse P2G, which follows, writes the v and C words without reading them
             float4 *op = aout + (size_t)p * ADJ_F4;
             op[0] = make_float4(xa[0], xa[1], xa[2], 0.f);
-            op[1] = make_float4(0.f, 0.f, 0.f, 0.f);
-            op[2] = make_float4(0.f, 0.f, 0.f, 0.f);
             op[3] = make_float4(0.f, 0.f, 0.f, Fp[0]);
             op[4] = make_float4(Fp[1], Fp[2], Fp[3], Fp[4]);
             op[5] = make_float4(Fp[5], Fp[6], Fp[7], Fp[8]);
-            float gE, gnu;
-            lame_chain(P.mu, P.lam, mubar, lambar, gE, gnu);
-            float4 g4 = gpar[p];
-            g4.x += gE; g4.y += gnu; g4.z += ybar;
-            gpar[p] = g4;
-            // packet for the scatter of the grid-velocity adjoint
-            // base cell (0..3 per axis) exactly in .w as 1 + b0 + 4 b1 + 16 b2 (> 0 marks a valid packet)
-            S.pk[tid * 4 + 0] = make_float4(f[0], f[1], f[2], (float)(1 + b[0] + 4 * b[1] + 16 * b[2]));
-            S.pk[tid * 4 + 1] = make_float4(vt[0], vt[1], vt[2], Ct[0]);
-            S.pk[tid * 4 + 2] = make_float4(Ct[1], Ct[2], Ct[3], Ct[4]);
-            S.pk[tid * 4 + 3] = make_float4(Ct[5], Ct[6], Ct[7], Ct[8]);
+            if (MS != ADJ_ELASTIC && (mubar != 0.f || lambar != 0.f || ybar != 0.f)) {
+                float gE, gnu;
+                lame_chain(P.mu, P.lam, mubar, lambar, gE, gnu);
+                float4 g4 = gpar[p];
+                g4.x += gE; g4.y += gnu; g4.z += ybar;
+                gpar[p] = g4;
+            }
             float cm = 0.f;
 #pragma unroll
             for (int t = 0; t < 9; ++t) cm = fmaxf(cm, fabsf(Ct[t]));
             bnd = fmaxf(fabsf(vt[0]), fmaxf(fabsf(vt[1]), fabsf(vt[2]))) + 4.5f * c4 * dx * cm;
-        } else {
-            S.pk[tid * 4] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
         // per-chunk fixed-point scale
 #pragma unroll
@@ -716,43 +708,39 @@ __global__ void __launch_bounds__(ADJ_THREADS, 3) k_adj_g2p(Dev D, const float4 
         __syncthreads();
         if (has_next) adj_stage3(D, S, S.cd[(kc + 1) % 3], ain, (kc + 1) & 1, ep);
         a_commit();
-        if (tid == 0) {
-            float bs = 0.f;
-            for (int wq = 0; wq < ADJ_THREADS / 32; ++wq) bs += S.red[wq];
-            S.scale = bs > 0.f ? 1073741824.f / bs : 1.f;
-        }
-        __syncthreads();
-        const float sc = S.scale;
-        // phase B: lane-transposed mapping spreads a warp over the chunk's cells
+        float bs = 0.f;
+#pragma unroll
+        for (int wq = 0; wq < ADJ_THREADS / 32; ++wq) bs += S.red[wq];
+        const float sc = bs > 0.f ? 1073741824.f / bs : 1.f;
+        // phase B: each thread its own particle, in list order
         {
-            const int j = (tid & 31) * (ADJ_THREADS / 32) + (tid >> 5);
-            const float4 q0 = S.pk[j * 4];
-            if (j < cnt && q0.w > 0.f) {
-                const float4 q1 = S.pk[j * 4 + 1], q2 = S.pk[j * 4 + 2], q3 = S.pk[j * 4 + 3];
-                const float vt[3] = {q1.x * sc, q1.y * sc, q1.z * sc};
-                const float Cs[9] = {q1.w * sc * c4 * dx, q2.x * sc * c4 * dx, q2.y * sc * c4 * dx,
-                                     q2.z * sc * c4 * dx, q2.w * sc * c4 * dx, q3.x * sc * c4 * dx,
-                                     q3.y * sc * c4 * dx, q3.z * sc * c4 * dx, q3.w * sc * c4 * dx};
-                const int code = (int)q0.w - 1;
-                const int b[3] = {code & 3, (code >> 2) & 3, (code >> 4) & 3};
-                const float f[3] = {q0.x, q0.y, q0.z};
+            if (valid) {
+                const float cs = sc * c4 * dx;
+                float Cs[9];
+#pragma unroll
+                for (int t = 0; t < 9; ++t) Cs[t] = Ct[t] * cs;
+#pragma unroll
+                for (int t = 0; t < 3; ++t) vt[t] *= sc;
                 float w[3][3];
 #pragma unroll
                 for (int a = 0; a < 3; ++a) bspline_w(f[a], w[a]);
 #pragma unroll 1
-                for (int i = 0; i < 3; ++i)
+                for (int i = 0; i < 3; ++i) {
+                    const float wi = i == 0 ? w[0][0] : (i == 1 ? w[0][1] : w[0][2]);   // selected, not indexed: registers
+                    const int ndi = gidx(b[0] + i, b[1], b[2]);
 #pragma unroll
                     for (int jj = 0; jj < 3; ++jj)
 #pragma unroll
                         for (int k = 0; k < 3; ++k) {
-                            const float wt = w[0][i] * w[1][jj] * w[2][k];
+                            const float wt = wi * w[1][jj] * w[2][k];
                             const float d[3] = {(float)i - f[0], (float)jj - f[1], (float)k - f[2]};
-                            const int node = gidx(b[0] + i, b[1] + jj, b[2] + k);
+                            const int node = ndi + jj * 8 + k;
 #pragma unroll
                             for (int r = 0; r < 3; ++r)
                                 atomicAdd(&S.t[r * GT3P + node],
                                           __float2int_rn(wt * (vt[r] + Cs[3 * r] * d[0] + Cs[3 * r + 1] * d[1] + Cs[3 * r + 2] * d[2])));
                         }
+                }
             }
         }
         __syncthreads();
@@ -818,7 +806,7 @@ __global__ void k_adj_grid(Dev D, float4 *gbar) {
 constexpr int PS_F4 = 13;                   // staged stride: record (8), adjoint words 0,3,4,5 (4), gpar (1)
 struct AdjP2GSmem {
     float4 st[ADJ_THREADS * PS_F4];
-    float4 g[GT3];                           // grid adjoint tile (Pbar, mbar)
+    float4 g[GTN];                           // grid adjoint tile (Pbar, mbar)
     int4 cd[3];
     unsigned pidx[ADJ_THREADS];
     unsigned pe[8];
@@ -844,8 +832,9 @@ __device__ __forceinline__ void adj_p2g_stage3(const Dev &D, AdjP2GSmem &S, int4
         const int i = t / (GT * GT), j = (t / GT) % GT, k = t % GT;
         const int b = ((i >> 2) << 2) | ((j >> 2) << 1) | (k >> 2);
         const int sl = S.pe[b] == ep ? S.ps[b] : -1;
-        if (sl >= 0) a_cp16(&S.g[t], gbar + (size_t)sl * BLK_NODES + node_loc(i, j, k));
-        else S.g[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+        const int q = gidx(i, j, k);
+        if (sl >= 0) a_cp16(&S.g[q], gbar + (size_t)sl * BLK_NODES + node_loc(i, j, k));
+        else S.g[q] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
 }
 
@@ -883,8 +872,8 @@ __global__ void __launch_bounds__(ADJ_THREADS, 3) k_adj_p2g(Dev D, float4 *aout,
         if (tid == 0 && cn + gridDim.x < n_chunks) a_cp16(&S.cd[(kc + 2) % 3], D.chunks + cn + gridDim.x);
         if (has_next) adj_stage2(D, S, S.cd[(kc + 1) % 3], ep);
         a_commit();
-        int inst, bx, by, bz;
-        key_coords(D, (unsigned)ch.x, inst, bx, by, bz);
+        int bx, by, bz;
+        item_coords(ch.w, bx, by, bz);
         bool ok = tid < cnt;
         float4 o0, o3, o4, o5, g4;
         float xa[3], va[3], Ab[9], Fb[9], mubar = 0.f, lambar = 0.f;
@@ -947,7 +936,7 @@ __global__ void __launch_bounds__(ADJ_THREADS, 3) k_adj_p2g(Dev D, float4 *aout,
                 const float wi = i == 0 ? w[0][0] : (i == 1 ? w[0][1] : w[0][2]);
                 const float dwi = i == 0 ? dw[0][0] : (i == 1 ? dw[0][1] : dw[0][2]);
                 const float di = ((float)i - f[0]) * dx;
-                const float4 *gi = S.g + (b[0] + i) * GT * GT;
+                const float4 *gi = S.g + gidx(b[0] + i, b[1], b[2]);
 #pragma unroll
                 for (int jj = 0; jj < 3; ++jj)
 #pragma unroll
@@ -956,7 +945,7 @@ __global__ void __launch_bounds__(ADJ_THREADS, 3) k_adj_p2g(Dev D, float4 *aout,
                         const float wt = wi * wjk;
                         const float gw[3] = {dwi * wjk, wi * dw[1][jj] * w[2][k], wi * w[1][jj] * dw[2][k]};
                         const float dp[3] = {di, ((float)jj - f[1]) * dx, ((float)k - f[2]) * dx};
-                        const float4 g = gi[(b[1] + jj) * GT + (b[2] + k)];
+                        const float4 g = gi[jj * 8 + k];
                         const float Pb[3] = {g.x, g.y, g.z};
                         float wbar = g.w * P.mass;
 #pragma unroll
