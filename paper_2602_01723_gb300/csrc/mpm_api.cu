@@ -252,7 +252,7 @@ void L_between(mpm_ctx *ctx, int upd, int act, cudaStream_t st) {
     ctx->bins_pending = false;
 }
 void L_substep(mpm_ctx *ctx, int mode, int gpar, int spar, cudaStream_t st, bool direct, int in_par,
-               int flags) {
+               int flags, float4 *rec_out) {
     cudaEvent_t *ev = nullptr;
     if (ctx->trace_on) {
         std::vector<cudaEvent_t> &pool = ctx->trace_ev[mode];
@@ -269,6 +269,7 @@ void L_substep(mpm_ctx *ctx, int mode, int gpar, int spar, cudaStream_t st, bool
         }
     }
     Dev Dc = ctx->D;
+    Dc.rec_out = rec_out ? rec_out : Dc.rec;
     if (in_par >= 0) {   // the work items and lists of the direct binning into buffer in_par
         Dc.chunks = ctx->D.chunksd[in_par];
         Dc.chunk_ctr = CTR_D_CH + in_par;

@@ -70,6 +70,7 @@ struct Dev {
     // particles
     int n;
     float4 *rec;           // n * REC_F4
+    float4 *rec_out;       // where a substep writes the records: rec, or the tape slot of the state it reaches
     // binning (current positions)
     unsigned *key;         // n
     unsigned *rank;        // n

@@ -742,7 +742,7 @@ __device__ __forceinline__ void stage_slots(SubstepSmem<TPB> &S, int buf, unsign
 // overwrites both before anything reads them, so a fused substep whose state
 // is not kept (no checkpoint, no tape) leaves them out; a run's last substep
 // writes them.
-// OWN (direct binning, fixed-point scatter): each thread scatters its own
+// OWN (fixed-point scatter): each thread scatters its own
 // particle from registers, in the order of the list, instead of handing
 // packets over in the (rank, bank) order.
 template <int MODE, int SCAT, int TPB, bool XM, bool DB, bool OWN>
@@ -842,7 +842,7 @@ __global__ void __launch_bounds__(TPB, 512 / TPB) k_substep(Dev D, int gpar, int
                 F[7] = r6.x; F[8] = r6.y;
                 Cm[8] = r4.x;
             }
-            float4 *rp = D.rec + (size_t)p * REC_F4;
+            float4 *rp = D.rec_out + (size_t)p * REC_F4;
             bool in_dom = true;
             int c0 = 0, c1 = 0, c2 = 0;   // the block of the new position
             if (GATHER) {
@@ -905,6 +905,7 @@ __global__ void __launch_bounds__(TPB, 512 / TPB) k_substep(Dev D, int gpar, int
                     rp[1] = make_float4(v[0], v[1], v[2], vol);
                     rp[2] = make_float4(Cm[0], Cm[1], Cm[2], Cm[3]);
                     rp[3] = make_float4(Cm[4], Cm[5], Cm[6], Cm[7]);
+                    if (!DB && D.rec_out != D.rec) rp[7] = r7;   // (what a substep does not change)
                 }
                 // F <- (I + dt C) F
                 float G[9];
@@ -1399,6 +1400,7 @@ static void launch_tpb(const Dev &D, int mode, int gpar, int spar, int grid, boo
     if (D.xm) {   // further models: the shared-memory fixed-point scatter only
         if (mode == MODE_G2P) launch_sub<MODE_G2P, 2, TPB, true>(D, gpar, spar, grid, keep, st);
         else if (mode == MODE_P2G) launch_sub<MODE_P2G, 1, TPB, true>(D, gpar, spar, grid, keep, st);
+        else if (own) launch_sub<MODE_FUSED, 1, TPB, true, false, true>(D, gpar, spar, grid, keep, st);
         else launch_sub<MODE_FUSED, 1, TPB, true>(D, gpar, spar, grid, keep, st);
         return;
     }
@@ -1410,8 +1412,9 @@ static void launch_tpb(const Dev &D, int mode, int gpar, int spar, int grid, boo
         return;
     }
     if (D.scatter == 0) launch_sub<MODE_FUSED, 0, TPB, false>(D, gpar, spar, grid, keep, st);
-    else if (D.scatter == 1) launch_sub<MODE_FUSED, 1, TPB, false>(D, gpar, spar, grid, keep, st);
-    else launch_sub<MODE_FUSED, 2, TPB, false>(D, gpar, spar, grid, keep, st);
+    else if (D.scatter == 2) launch_sub<MODE_FUSED, 2, TPB, false>(D, gpar, spar, grid, keep, st);
+    else if (own) launch_sub<MODE_FUSED, 1, TPB, false, false, true>(D, gpar, spar, grid, keep, st);
+    else launch_sub<MODE_FUSED, 1, TPB, false>(D, gpar, spar, grid, keep, st);
 }
 // the chunk size selects the CTA size: chunks of <= 64 particles run 64-thread CTAs
 void launch_substep(const Dev &D, int mode, int gpar, int spar, int grid, bool direct, int flags, cudaStream_t st) {
@@ -1437,9 +1440,12 @@ template <int MODE, int SCAT, int TPB, bool XM> static int occ_of() {
     if constexpr (MODE == MODE_FUSED && SCAT != 0)   // its direct-binning variants
         cudaFuncSetAttribute(k_substep<MODE, SCAT, TPB, XM, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)substep_smem<TPB, false>());
-    if constexpr (MODE == MODE_FUSED && SCAT == 1)
+    if constexpr (MODE == MODE_FUSED && SCAT == 1) {
+        cudaFuncSetAttribute(k_substep<MODE, SCAT, TPB, XM, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)substep_smem<TPB, true>());
         cudaFuncSetAttribute(k_substep<MODE, SCAT, TPB, XM, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)substep_smem<TPB, true>());
+    }
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_substep<MODE, SCAT, TPB, XM, false, false>, TPB,
                                                   substep_smem<TPB, false>());
     return nb;

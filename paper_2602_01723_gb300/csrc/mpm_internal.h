@@ -49,7 +49,7 @@ void launch_bin(const Dev &D, cudaStream_t st);
 void launch_plan(const Dev &D, int bump_mask, cudaStream_t st);
 void launch_prepare(const Dev &D, int upd_par, int act_par, int do_sort, int keep_momentum, int grid, cudaStream_t st);
 // flags of the fused mode: SUB_KEEP writes v and C to the records, SUB_OWN
-// (direct binning, fixed-point scatter) scatters in list order (see k_substep)
+// (fixed-point scatter) scatters in list order (see k_substep)
 enum { SUB_KEEP = 1, SUB_OWN = 2 };
 // direct: the fused mode bins straight into the scatter buffer's lists
 void launch_substep(const Dev &D, int mode, int gpar, int spar, int grid, bool direct, int flags, cudaStream_t st);
@@ -187,9 +187,11 @@ void L_plan(mpm_ctx *ctx, int bump_mask, cudaStream_t st);
 // grid update of upd_par, activation of act_par, sorted index (see k_prepare)
 void L_prepare(mpm_ctx *ctx, int upd_par, int act_par, int do_sort, cudaStream_t st, int keep_momentum = 0);
 // direct: bin straight into the scatter buffer's lists (fused mode); in_par
-// >= 0: read the work items of the direct binning into buffer in_par
+// >= 0: read the work items of the direct binning into buffer in_par;
+// rec_out: write the new records there, in place of the state's (fused mode
+// with a sort, SUB_KEEP)
 void L_substep(mpm_ctx *ctx, int mode, int gpar, int spar, cudaStream_t st, bool direct = false, int in_par = -1,
-               int flags = SUB_KEEP);
+               int flags = SUB_KEEP, float4 *rec_out = nullptr);
 void L_between(mpm_ctx *ctx, int upd, int act, cudaStream_t st);
 void L_bin(mpm_ctx *ctx, cudaStream_t st);
 void launch_bgdo_accum(const Dev &D, const float4 *key, const float4 *post, int first, float inv_k,
