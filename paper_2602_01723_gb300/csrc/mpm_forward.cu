@@ -741,7 +741,7 @@ __device__ __forceinline__ void stage_slots(SubstepSmem<TPB> &S, int buf, unsign
 // keep: the new v and C go to the particle's record too.  The next gather
 // overwrites both before anything reads them, so a fused substep whose state
 // is not kept (no checkpoint, no tape) leaves them out; a run's last substep
-// writes them.
+// (G2P) writes them and, with keep, bins the particles for what follows.
 // OWN (fixed-point scatter): each thread scatters its own
 // particle from registers, in the order of the list, instead of handing
 // packets over in the (rank, bank) order.
@@ -899,7 +899,8 @@ __global__ void __launch_bounds__(TPB, 512 / TPB) k_substep(Dev D, int gpar, int
                 if (!(isfinite(vn[0]) && isfinite(vn[1]) && isfinite(vn[2]))) set_err(D, ERRB_NONFINITE);
                 if (!ORDERED) {   // the atomic's result is consumed after the SVD
                     in_dom = particle_block(D, q[0], q[1], q[2], c0, c1, c2);
-                    ticket = bin_begin(D, lane_mask, key_offset(D, (unsigned)ch.x, c0 - bx, c1 - by, c2 - bz));
+                    if (MODE != MODE_G2P || keep)
+                        ticket = bin_begin(D, lane_mask, key_offset(D, (unsigned)ch.x, c0 - bx, c1 - by, c2 - bz));
                 }
                 if (MODE == MODE_G2P || keep) {
                     rp[1] = make_float4(v[0], v[1], v[2], vol);
@@ -1050,7 +1051,7 @@ __global__ void __launch_bounds__(TPB, 512 / TPB) k_substep(Dev D, int gpar, int
                                     __uint_as_float(key_offset(D, (unsigned)ch.x, c0 - bx, c1 - by, c2 - bz)), 0.f);
                 }
             }
-            if (!ORDERED && MODE != MODE_P2G)
+            if (!ORDERED && MODE != MODE_P2G && (MODE != MODE_G2P || keep))
                 entry = DB ? bin_end_direct(D, ticket, p, slot, spar) : bin_end(D, ticket, p);
             }
         }

@@ -48,7 +48,8 @@ void launch_load(const Dev &D, const LoadArgs &a, cudaStream_t st);   // bins th
 void launch_bin(const Dev &D, cudaStream_t st);
 void launch_plan(const Dev &D, int bump_mask, cudaStream_t st);
 void launch_prepare(const Dev &D, int upd_par, int act_par, int do_sort, int keep_momentum, int grid, cudaStream_t st);
-// flags of the fused mode: SUB_KEEP writes v and C to the records, SUB_OWN
+// flags: SUB_KEEP writes v and C to the records (fused mode; G2P always does)
+// and bins the new state (G2P; the fused mode always does), SUB_OWN
 // (fixed-point scatter) scatters in list order (see k_substep)
 enum { SUB_KEEP = 1, SUB_OWN = 2 };
 // direct: the fused mode bins straight into the scatter buffer's lists
@@ -188,8 +189,8 @@ void L_plan(mpm_ctx *ctx, int bump_mask, cudaStream_t st);
 void L_prepare(mpm_ctx *ctx, int upd_par, int act_par, int do_sort, cudaStream_t st, int keep_momentum = 0);
 // direct: bin straight into the scatter buffer's lists (fused mode); in_par
 // >= 0: read the work items of the direct binning into buffer in_par;
-// rec_out: write the new records there, in place of the state's (fused mode
-// with a sort, SUB_KEEP)
+// rec_out: write the new records there and leave the state's as they are
+// (G2P, or the fused mode with a sort and SUB_KEEP)
 void L_substep(mpm_ctx *ctx, int mode, int gpar, int spar, cudaStream_t st, bool direct = false, int in_par = -1,
                int flags = SUB_KEEP, float4 *rec_out = nullptr);
 void L_between(mpm_ctx *ctx, int upd, int act, cudaStream_t st);
