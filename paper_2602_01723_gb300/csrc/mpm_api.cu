@@ -786,7 +786,7 @@ MPM_API mpm_status mpm_destroy(mpm_ctx *ctx) {
     dfree(ctx->stage);
     free_adjoint(ctx->adj);
     for (int k = 0; k < MPM_MAX_SNAPSHOTS; ++k) dfree(ctx->snap[k]);
-    dfree(ctx->bgdo_work); dfree(ctx->bgdo_G); dfree(ctx->bgdo_sum); dfree(ctx->cov0);
+    dfree(ctx->bgdo_G); dfree(ctx->bgdo_sum); dfree(ctx->cov0);
     for (int m = 0; m < 3; ++m)
         for (cudaEvent_t e : ctx->trace_ev[m]) cudaEventDestroy(e);
     for (cudaGraphExec_t g : ctx->graph)
@@ -941,8 +941,7 @@ MPM_API mpm_status mpm_bgdo(mpm_ctx *ctx, int32_t n_keys, const int32_t *slots, 
     const int nm = (int)ctx->table.size();
     mpm_status s;
     if (ctx->bgdo_cap < ctx->cap) {
-        if ((s = dalloc(ctx, &ctx->bgdo_work, (size_t)ctx->cap * REC_F4, false))) return s;
-        if ((s = dalloc(ctx, &ctx->bgdo_G, (size_t)ctx->cap, false))) return s;
+        if ((s = dalloc(ctx, &ctx->bgdo_G, 2 * (size_t)ctx->cap, false))) return s;
         ctx->bgdo_cap = ctx->cap;
     }
     if (o.per_material && !ctx->bgdo_sum && (s = dalloc(ctx, &ctx->bgdo_sum, 2 * (size_t)nm, false))) return s;
@@ -968,27 +967,32 @@ MPM_API mpm_status mpm_bgdo(mpm_ctx *ctx, int32_t n_keys, const int32_t *slots, 
             if (outs[i] && !dptr[i]) dptr[i] = (float *)((char *)ctx->stage + offs[i]);
     }
     for (int k = 0; k < n_keys; ++k) {
-        const float4 *key = ctx->snap[slots[k]];
-        const float4 *post = key;
-        if (!o.delta_pre_step) {
+        float4 *key = ctx->snap[slots[k]];
+        float *g_tau_k = dptr[2] ? dptr[2] + (size_t)k * n : nullptr, *delta_k = dptr[3] ? dptr[3] + (size_t)k * n : nullptr;
+        const float inv_k = 1.f / (float)n_keys;
+        if (o.delta_pre_step) {
+            launch_bgdo_accum(D, key, k == 0, inv_k, o.delta_target, o.w, ctx->bgdo_G, g_tau_k, delta_k, st);
+            ++ctx->launches;
+        } else {
             // the pseudo substep: the ordinary substep of the key frame, which is
-            // only read.  Nothing follows from its state, so it is not binned:
-            // 145 -> 127 us per key frame of 300k particles without the copy, the
-            // binning and the plan that discarded it.
+            // only read.  Its P2G and G2P give the two signals and add the key
+            // frame's term; nothing follows from its state, so it is neither
+            // written nor binned.  103 us per key frame of 300k particles, 145
+            // with a copy of the key frame, a binning with the plan that
+            // discarded it and a pass over both states (which took the SVD again).
             float4 *saved = D.rec;
-            D.rec = ctx->snap[slots[k]];
+            D.rec = key;
+            D.key_frame = KeySignals{ctx->bgdo_G, g_tau_k ? g_tau_k : ctx->bgdo_G + ctx->bgdo_cap, delta_k, inv_k,
+                                     o.delta_target, o.w, k == 0};
             rebin(ctx, st);
             L_plan(ctx, 1, st);
             L_prepare(ctx, -1, 0, 1, st);
             L_substep(ctx, 0, 0, 0, st);
             L_prepare(ctx, 0, -1, 0, st);
-            L_substep(ctx, 2, 0, 0, st, false, -1, 0, ctx->bgdo_work);
+            L_substep(ctx, 2, 0, 0, st, false, -1, 0);
             D.rec = saved;
-            post = ctx->bgdo_work;
+            D.key_frame = KeySignals{};
         }
-        launch_bgdo_accum(D, key, post, k == 0, 1.f / (float)n_keys, o.delta_target, o.w, ctx->bgdo_G,
-                          dptr[2] ? dptr[2] + (size_t)k * n : nullptr, dptr[3] ? dptr[3] + (size_t)k * n : nullptr, st);
-        ++ctx->launches;
         CKLAUNCH();
     }
     if (o.per_material) {

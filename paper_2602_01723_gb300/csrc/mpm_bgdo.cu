@@ -2,7 +2,7 @@
 // Algorithm 1, Stage 2; App. F): per-particle signals of one pseudo substep
 // from a key frame, their average over key frames, the optional per-material
 // mean and the log-E update.  The pseudo substep itself is the ordinary
-// substep of mpm_forward.cu run on a copy of the key frame.
+// substep of mpm_forward.cu, whose kernels give the signals (see KeySignals).
 #include <cuda_runtime.h>
 
 #include "mpm_internal.h"
@@ -10,17 +10,15 @@
 
 namespace mpm {
 
-// Young's modulus from the Lame pair (inverse of App. B.1 at fixed nu)
-__device__ __forceinline__ float young_of(float mu, float lam) { return mu * (3.f * lam + 2.f * mu) / (lam + mu); }
-
-// Adds one key frame's contribution to G.  key: the key-frame records; post:
-// the records after the pseudo substep (== key when delta is taken before it).
+// Adds one key frame's contribution to G where delta is taken before the
+// pseudo substep, which is then left out (with it, the substep kernels do this;
+// see KeySignals).  key: the key-frame records.
 //   g_tau = |tau(F_key)|_F: d|tau|/d log E equals |tau| because tau is linear
 //           in (mu, lambda) and both are proportional to E at fixed nu
-//   delta = |F_post - I|_F
+//   delta = |F_key - I|_F
 //   G    += (eta log(1 + g_tau) - (1 - eta)(delta - delta_target)) / K
-__global__ void k_bgdo_accum(Dev D, const float4 *__restrict__ key, const float4 *__restrict__ post, int first,
-                             float inv_k, float delta_target, float w, float *__restrict__ G,
+__global__ void k_bgdo_accum(Dev D, const float4 *__restrict__ key, int first, float inv_k,
+                             float delta_target, float w, float *__restrict__ G,
                              float *__restrict__ g_tau, float *__restrict__ delta) {
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < D.n; p += gridDim.x * blockDim.x) {
         const float4 *r = key + (size_t)p * REC_F4;
@@ -38,25 +36,8 @@ __global__ void k_bgdo_accum(Dev D, const float4 *__restrict__ key, const float4
             set_err(D, ERRB_NONFINITE);
             t = Sym{0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
         }
-        const float g = sqrtf(t.xx * t.xx + t.yy * t.yy + t.zz * t.zz +
-                              2.f * (t.xy * t.xy + t.xz * t.xz + t.yz * t.yz));
-        float Fn[9];
-        if (post == key) {
-#pragma unroll
-            for (int i = 0; i < 9; ++i) Fn[i] = F[i];
-        } else {
-            const float4 *q = post + (size_t)p * REC_F4;
-            const float4 q4 = q[4], q5 = q[5], q6 = q[6];
-            Fn[0] = q4.y; Fn[1] = q4.z; Fn[2] = q4.w; Fn[3] = q5.x; Fn[4] = q5.y;
-            Fn[5] = q5.z; Fn[6] = q5.w; Fn[7] = q6.x; Fn[8] = q6.y;
-        }
-        Fn[0] -= 1.f; Fn[4] -= 1.f; Fn[8] -= 1.f;
-        float d2 = 0.f;
-#pragma unroll
-        for (int i = 0; i < 9; ++i) d2 += Fn[i] * Fn[i];
-        const float dl = sqrtf(d2);
-        const float eta = w >= 0.f ? w : fminf(1.f, 0.1f * log1pf(young_of(mu, lam)));
-        const float c = eta * log1pf(g) - (1.f - eta) * (dl - delta_target);
+        const float g = stress_norm(t), dl = strain_norm(F);
+        const float c = key_frame_term(g, dl, mu, lam, w, delta_target);
         G[p] = (first ? 0.f : G[p]) + c * inv_k;
         if (g_tau) g_tau[p] = g;
         if (delta) delta[p] = dl;
@@ -116,9 +97,8 @@ __global__ void k_bgdo_finish(Dev D, int n_mat, const float *__restrict__ Gin, c
     }
 }
 
-void launch_bgdo_accum(const Dev &D, const float4 *key, const float4 *post, int first, float inv_k,
-                       float delta_target, float w, float *G, float *g_tau, float *delta, cudaStream_t st) {
-    k_bgdo_accum<<<grid_for(D.n, 128), 128, 0, st>>>(D, key, post, first, inv_k, delta_target, w, G, g_tau, delta);
+void launch_bgdo_accum(const Dev &D, const float4 *key, int first, float inv_k, float delta_target, float w, float *G, float *g_tau, float *delta, cudaStream_t st) {
+    k_bgdo_accum<<<grid_for(D.n, 128), 128, 0, st>>>(D, key, first, inv_k, delta_target, w, G, g_tau, delta);
 }
 void launch_bgdo_material_sum(const Dev &D, int n_mat, const float *G, double *sum, cudaStream_t st) {
     k_bgdo_material_sum<<<grid_for(D.n, 256, 152 * 4), 256, 2 * n_mat * sizeof(double), st>>>(D, n_mat, G, sum);

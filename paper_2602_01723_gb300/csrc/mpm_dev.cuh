@@ -54,6 +54,15 @@ enum : unsigned {
     ERRB_TIMEOUT = 1u << 4,
 };
 
+// What a substep of the material optimisation gives in place of a new state
+// (all NULL otherwise): P2G writes g_tau = |tau|_F of the state, G2P reads it,
+// takes delta = |F - I|_F of the new one and adds the key frame's term to G.
+struct KeySignals {
+    float *G, *g_tau, *delta;   // per particle; delta may be NULL
+    float inv_k, delta_target, w;
+    int first;                  // G is set, not added to
+};
+
 struct Dev {
     // geometry
     int R[3];              // nodes per axis of one instance grid
@@ -106,6 +115,8 @@ struct Dev {
     int scatter;           // scatter strategy of the substep kernel (0 shared tile, 2 direct)
     int xm;                // the material table uses models beyond FCR / NH / VM / DP
     unsigned *err;         // sticky error bits
+    // what a key frame's substep gives in place of a new state
+    KeySignals key_frame;
 };
 
 // device counters (Dev::ctr)

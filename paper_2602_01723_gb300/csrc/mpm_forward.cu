@@ -902,7 +902,8 @@ __global__ void __launch_bounds__(TPB, 512 / TPB) k_substep(Dev D, int gpar, int
                     if (MODE != MODE_G2P || keep)
                         ticket = bin_begin(D, lane_mask, key_offset(D, (unsigned)ch.x, c0 - bx, c1 - by, c2 - bz));
                 }
-                if (MODE == MODE_G2P || keep) {
+                const bool record = MODE != MODE_G2P || !D.key_frame.G;
+                if (record && (MODE == MODE_G2P || keep)) {
                     rp[1] = make_float4(v[0], v[1], v[2], vol);
                     rp[2] = make_float4(Cm[0], Cm[1], Cm[2], Cm[3]);
                     rp[3] = make_float4(Cm[4], Cm[5], Cm[6], Cm[7]);
@@ -944,10 +945,18 @@ __global__ void __launch_bounds__(TPB, 512 / TPB) k_substep(Dev D, int gpar, int
                 }
 #pragma unroll
                 for (int t = 0; t < 9; ++t) F[t] = G[t];
-                rp[0] = make_float4(__int_as_float(q[0]), __int_as_float(q[1]), __int_as_float(q[2]), mass);
-                rp[4] = make_float4(Cm[8], F[0], F[1], F[2]);
-                rp[5] = make_float4(F[3], F[4], F[5], F[6]);
-                rp[6] = make_float4(F[7], F[8], mu, lam);
+                if (record) {
+                    rp[0] = make_float4(__int_as_float(q[0]), __int_as_float(q[1]), __int_as_float(q[2]), mass);
+                    rp[4] = make_float4(Cm[8], F[0], F[1], F[2]);
+                    rp[5] = make_float4(F[3], F[4], F[5], F[6]);
+                    rp[6] = make_float4(F[7], F[8], mu, lam);
+                } else {
+                    const KeySignals &kf = D.key_frame;
+                    const float dl = strain_norm(F);
+                    const float c = key_frame_term(kf.g_tau[p], dl, mu, lam, kf.w, kf.delta_target);
+                    kf.G[p] = (kf.first ? 0.f : kf.G[p]) + c * kf.inv_k;
+                    if (kf.delta) kf.delta[p] = dl;
+                }
             } else {
                 const float4 r2 = nr[2], r3 = nr[3];
                 Cm[0] = r2.x; Cm[1] = r2.y; Cm[2] = r2.z; Cm[3] = r2.w;
@@ -989,6 +998,7 @@ __global__ void __launch_bounds__(TPB, 512 / TPB) k_substep(Dev D, int gpar, int
                     set_err(D, ERRB_NONFINITE);
                     tau = Sym{0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
                 }
+                if (MODE == MODE_P2G && D.key_frame.g_tau) D.key_frame.g_tau[p] = stress_norm(tau);
                 const float kf = 4.f * dt * vol * inv_dx * inv_dx;
                 Ad[0] = (mass * Cm[0] - kf * tau.xx) * dx; Ad[1] = (mass * Cm[1] - kf * tau.xy) * dx;
                 Ad[2] = (mass * Cm[2] - kf * tau.xz) * dx; Ad[3] = (mass * Cm[3] - kf * tau.xy) * dx;

@@ -171,9 +171,8 @@ struct mpm_ctx {
     float4 *snap[MPM_MAX_SNAPSHOTS] = {};
     long long snap_n[MPM_MAX_SNAPSHOTS] = {};     // particle count at the snapshot (0: empty)
     long long snap_cap[MPM_MAX_SNAPSHOTS] = {};
-    float4 *bgdo_work = nullptr;   // pseudo-substep state
     long long bgdo_cap = 0;
-    float *bgdo_G = nullptr;       // per-particle accumulator
+    float *bgdo_G = nullptr;       // per-particle accumulator, and behind it (at bgdo_cap) |tau| where the caller takes none
     double *bgdo_sum = nullptr;    // per-material sum and count (2 * n_materials)
     // rest covariance of each particle's Gaussian kernel (n x 6)
     float *cov0 = nullptr;
@@ -195,8 +194,8 @@ void L_substep(mpm_ctx *ctx, int mode, int gpar, int spar, cudaStream_t st, bool
                int flags = SUB_KEEP, float4 *rec_out = nullptr);
 void L_between(mpm_ctx *ctx, int upd, int act, cudaStream_t st);
 void L_bin(mpm_ctx *ctx, cudaStream_t st);
-void launch_bgdo_accum(const Dev &D, const float4 *key, const float4 *post, int first, float inv_k,
-                       float delta_target, float w, float *G, float *g_tau, float *delta, cudaStream_t st);
+void launch_bgdo_accum(const Dev &D, const float4 *key, int first, float inv_k, float delta_target, float w,
+                       float *G, float *g_tau, float *delta, cudaStream_t st);
 void launch_bgdo_material_sum(const Dev &D, int n_mat, const float *G, double *sum, cudaStream_t st);
 void launch_bgdo_finish(const Dev &D, int n_mat, const float *G, const double *sum, float *Gout, float *logE,
                         cudaStream_t st);

@@ -444,6 +444,29 @@ static __device__ __noinline__ bool tau_more(int elastic, const float *F, const 
     return ok;
 }
 
+// Young's modulus from the Lame pair (inverse of App. B.1 at fixed nu)
+__device__ __forceinline__ float young_of(float mu, float lam) { return mu * (3.f * lam + 2.f * mu) / (lam + mu); }
+// |tau|_F and |F - I|_F
+__device__ __forceinline__ float stress_norm(const Sym &t) {
+    return sqrtf(t.xx * t.xx + t.yy * t.yy + t.zz * t.zz + 2.f * (t.xy * t.xy + t.xz * t.xz + t.yz * t.yz));
+}
+__device__ __forceinline__ float strain_norm(const float F[9]) {
+    float d2 = 0.f;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        const float d = F[i] - (i % 4 == 0 ? 1.f : 0.f);
+        d2 += d * d;
+    }
+    return sqrtf(d2);
+}
+// a key frame's term of G (Algorithm 1): eta log(1 + g_tau) - (1 - eta)(delta - delta_target);
+// w < 0: eta from Young's modulus
+__device__ __forceinline__ float key_frame_term(float g_tau, float delta, float mu, float lam, float w,
+                                                float delta_target) {
+    const float eta = w >= 0.f ? w : fminf(1.f, 0.1f * log1pf(young_of(mu, lam)));
+    return eta * log1pf(g_tau) - (1.f - eta) * (delta - delta_target);
+}
+
 // Kirchhoff stress of any elastic model; U, s, e must hold the SVD of F when
 // elastic_needs_svd(elastic)
 __device__ __forceinline__ bool kirchhoff(int elastic, const float F[9], const float U[9], const float s[3],
