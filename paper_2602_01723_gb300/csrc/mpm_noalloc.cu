@@ -70,7 +70,23 @@ __device__ __forceinline__ bool locate(const Params &P, const float *x, int b[3]
     return ok;
 }
 
+// The substep is four dependent launches of a few microseconds: at 8k particles
+// on 32^3 their latency counts, not the work.  Each but the first is a
+// programmatic dependent launch: it starts when every CTA of the one before has
+// started, loads its inputs and does what needs nothing of that one, and waits
+// for its end before it touches the grid or the error word.  The clear, launched
+// the ordinary way, starts after all earlier work of the stream, so the inputs are
+// there; each kernel waits in every thread, so the end of one implies that of all
+// before it, and outputs that alias inputs are written after all have read them.
+// CTAs of 64 particles: 8k particles then use 128 SMs, with 256 they used 32.
+// A call at 8k particles: 52.3 -> 43.0 us (44.3 with CTAs of 256), of which the
+// host's checks and launches and the read of the error word are some 25.
+constexpr int NA_T = 64;
+__device__ __forceinline__ void let_next_start() { cudaTriggerProgrammaticLaunchCompletion(); }
+__device__ __forceinline__ void wait_for_previous() { cudaGridDependencySynchronize(); }
+
 __global__ void k_na_clear(float4 *grid, unsigned *err, int nodes) {
+    let_next_start();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i == 0) err[0] = 0u;
     for (; i < nodes; i += gridDim.x * blockDim.x) grid[i] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -78,17 +94,26 @@ __global__ void k_na_clear(float4 *grid, unsigned *err, int nodes) {
 
 // P2G with the stress of F (the momentum equation of §4.2), straight into the
 // dense scratch grid with vector reductions
-__global__ void k_na_p2g(Params P, float4 *grid, unsigned *err, const float *__restrict__ x,
-                         const float *__restrict__ v, const float *__restrict__ C, const float *__restrict__ F,
-                         const float *__restrict__ vol, const int *__restrict__ mat) {
-    int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= P.n) return;
-    int m = mat[p];
-    if (m < 0 || m >= P.n_mat) { atomicOr(err, ERRB_DOMAIN); return; }
-    float xp[3] = {x[3 * p], x[3 * p + 1], x[3 * p + 2]};
+__global__ void __launch_bounds__(NA_T) k_na_p2g(Params P, float4 *grid, unsigned *err, const float *__restrict__ x,
+                                                const float *__restrict__ v, const float *__restrict__ C,
+                                                const float *__restrict__ F, const float *__restrict__ vol,
+                                                const int *__restrict__ mat) {
+    let_next_start();
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    const int m = p < P.n ? mat[p] : -1;
+    float xp[3] = {0.f, 0.f, 0.f};
     int b[3];
     float f[3];
-    if (!locate(P, xp, b, f)) { atomicOr(err, ERRB_DOMAIN); return; }
+    bool ok = p < P.n && m >= 0 && m < P.n_mat;
+    if (ok) {
+        xp[0] = x[3 * p]; xp[1] = x[3 * p + 1]; xp[2] = x[3 * p + 2];
+        ok = locate(P, xp, b, f);
+    }
+    if (!ok) {
+        wait_for_previous();
+        if (p < P.n) atomicOr(err, ERRB_DOMAIN);
+        return;
+    }
     float Fm[9], Cm[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) { Fm[i] = F[9 * p + i]; Cm[i] = C[9 * p + i]; }
@@ -96,12 +121,13 @@ __global__ void k_na_p2g(Params P, float4 *grid, unsigned *err, const float *__r
     const float mu = E / (2.f * (1.f + nu)), lam = E * nu / ((1.f + nu) * (1.f - 2.f * nu));
     const float mass = P.rho[m] * vol[p];
     Sym tau;
+    bool finite = true;
     if (P.elastic[m] == 0) {
         float U[9], V[9], s[3], e[3], d[3];
-        if (svd3_robust(Fm, U, V, s, e, d) == 2) atomicOr(err, ERRB_NONFINITE);
+        finite = svd3_robust(Fm, U, V, s, e, d) != 2;
         tau = tau_fcr(U, s, e, mu, lam);
     } else if (!tau_nh(Fm, mu, lam, tau)) {
-        atomicOr(err, ERRB_NONFINITE);
+        finite = false;
         tau = Sym{0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     }
     const float kf = 4.f * P.dt * vol[p] * P.inv_dx * P.inv_dx;
@@ -115,6 +141,8 @@ __global__ void k_na_p2g(Params P, float4 *grid, unsigned *err, const float *__r
     bspline_w(f[0], w0);
     bspline_w(f[1], w1);
     bspline_w(f[2], w2);
+    wait_for_previous();   // the grid and the error word are cleared
+    if (!finite) atomicOr(err, ERRB_NONFINITE);
     for (int i = 0; i < 3; ++i)
         for (int j = 0; j < 3; ++j)
             for (int k = 0; k < 3; ++k) {
@@ -129,6 +157,8 @@ __global__ void k_na_p2g(Params P, float4 *grid, unsigned *err, const float *__r
 
 // grid update (App. A): v = mv/m + dt g, then the walls, in place
 __global__ void k_na_update(Params P, float4 *grid, int nodes) {
+    let_next_start();
+    wait_for_previous();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nodes; i += gridDim.x * blockDim.x) {
         float4 a = grid[i];
         if (!(a.w > 0.f)) { grid[i] = make_float4(0.f, 0.f, 0.f, 0.f); continue; }
@@ -150,16 +180,20 @@ __global__ void k_na_update(Params P, float4 *grid, int nodes) {
 }
 
 // G2P, advection, F update and return map (App. A; Algorithm 1, Stage 1)
-__global__ void k_na_g2p(Params P, const float4 *grid, unsigned *err, const float *x, const float *F,
-                         const int *__restrict__ mat, float *x_out, float *v_out, float *C_out, float *F_out) {
-    int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= P.n) return;
-    int m = mat[p];
-    if (m < 0 || m >= P.n_mat) return;
-    float xp[3] = {x[3 * p], x[3 * p + 1], x[3 * p + 2]};
+__global__ void __launch_bounds__(NA_T) k_na_g2p(Params P, const float4 *grid, unsigned *err, const float *x,
+                                                const float *F, const int *__restrict__ mat, float *x_out,
+                                                float *v_out, float *C_out, float *F_out) {
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    const int m = p < P.n ? mat[p] : -1;
+    float xp[3] = {0.f, 0.f, 0.f};
     int b[3];
     float f[3];
-    if (!locate(P, xp, b, f)) return;
+    bool ok = m >= 0 && m < P.n_mat;
+    if (ok) {
+        xp[0] = x[3 * p]; xp[1] = x[3 * p + 1]; xp[2] = x[3 * p + 2];
+        ok = locate(P, xp, b, f);
+    }
+    if (!ok) { wait_for_previous(); return; }   // (P2G has reported it)
     float Fm[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) Fm[i] = F[9 * p + i];
@@ -168,18 +202,35 @@ __global__ void k_na_g2p(Params P, const float4 *grid, unsigned *err, const floa
     bspline_w(f[1], w1);
     bspline_w(f[2], w2);
     float vn[3] = {0.f, 0.f, 0.f}, Bm[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    for (int i = 0; i < 3; ++i)
-        for (int j = 0; j < 3; ++j)
+    wait_for_previous();   // the grid holds velocities
+    // separable sums, as in k_substep
+    const float wz1[3] = {w2[0] * (0.f - f[2]), w2[1] * (1.f - f[2]), w2[2] * (2.f - f[2])};
+    const float4 *gp = grid + (b[0] * P.R[1] + b[1]) * P.R[2] + b[2];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        float Ui[3] = {0.f, 0.f, 0.f}, Vi[3] = {0.f, 0.f, 0.f}, Wi[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            float Sij[3] = {0.f, 0.f, 0.f}, Tij[3] = {0.f, 0.f, 0.f};
+#pragma unroll
             for (int k = 0; k < 3; ++k) {
-                const float wt = w0[i] * w1[j] * w2[k];
-                const float d[3] = {(float)i - f[0], (float)j - f[1], (float)k - f[2]};
-                const float4 g = grid[((b[0] + i) * P.R[1] + (b[1] + j)) * P.R[2] + (b[2] + k)];
-                const float a[3] = {wt * g.x, wt * g.y, wt * g.z};
-                for (int r = 0; r < 3; ++r) {
-                    vn[r] += a[r];
-                    for (int c = 0; c < 3; ++c) Bm[3 * r + c] += a[r] * d[c];
-                }
+                const float4 g = gp[(i * P.R[1] + j) * P.R[2] + k];
+                Sij[0] += w2[k] * g.x; Sij[1] += w2[k] * g.y; Sij[2] += w2[k] * g.z;
+                Tij[0] += wz1[k] * g.x; Tij[1] += wz1[k] * g.y; Tij[2] += wz1[k] * g.z;
             }
+            const float wj = w1[j], wjd = w1[j] * ((float)j - f[1]);
+#pragma unroll
+            for (int r = 0; r < 3; ++r) { Ui[r] += wj * Sij[r]; Vi[r] += wjd * Sij[r]; Wi[r] += wj * Tij[r]; }
+        }
+        const float wi = w0[i], wid = w0[i] * ((float)i - f[0]);
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            vn[r] += wi * Ui[r];
+            Bm[3 * r] += wid * Ui[r];
+            Bm[3 * r + 1] += wi * Vi[r];
+            Bm[3 * r + 2] += wi * Wi[r];
+        }
+    }
     float Cn[9], G[9];
     for (int t = 0; t < 9; ++t) Cn[t] = 4.f * P.inv_dx * Bm[t];
     for (int r = 0; r < 3; ++r)
@@ -200,6 +251,21 @@ __global__ void k_na_g2p(Params P, const float4 *grid, unsigned *err, const floa
         v_out[3 * p + r] = vn[r];
     }
     for (int t = 0; t < 9; ++t) { C_out[9 * p + t] = Cn[t]; F_out[9 * p + t] = G[t]; }
+}
+
+// a launch that may start before the previous one in the stream has ended
+template <typename... Params_, typename... Args>
+cudaError_t launch_dependent(void (*kernel)(Params_...), int grid, int block, cudaStream_t st, Args... args) {
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, Params_(args)...);
 }
 
 }  // namespace
@@ -276,13 +342,17 @@ extern "C" MPM_API mpm_status mpm_substep_noalloc(const int32_t grid_res[3], flo
     }
     cudaStream_t st = (cudaStream_t)stream;
     const int nn = (int)nodes;
-    const int pgrid = (int)((n + 255) / 256);
+    const int pgrid = (int)((n + NA_T - 1) / NA_T);
     const int ggrid = (nn + 255) / 256 < 4096 ? (nn + 255) / 256 : 4096;
     k_na_clear<<<ggrid, 256, 0, st>>>(sc.grid, sc.err, nn);
-    k_na_p2g<<<pgrid, 256, 0, st>>>(P, sc.grid, sc.err, x, v, C, F, vol, material_id);
-    k_na_update<<<ggrid, 256, 0, st>>>(P, sc.grid, nn);
-    k_na_g2p<<<pgrid, 256, 0, st>>>(P, sc.grid, sc.err, x, F, material_id, x_out, v_out, C_out, F_out);
-    if (cudaGetLastError() != cudaSuccess) return MPM_ERR_CUDA;
+    if (cudaGetLastError() != cudaSuccess ||
+        launch_dependent(k_na_p2g, pgrid, NA_T, st, P, sc.grid, sc.err, x, v, C, F, vol, material_id) != cudaSuccess ||
+        launch_dependent(k_na_update, ggrid, 256, st, P, sc.grid, nn) != cudaSuccess ||
+        launch_dependent(k_na_g2p, pgrid, NA_T, st, P, sc.grid, sc.err, x, F, material_id, x_out, v_out, C_out, F_out) !=
+            cudaSuccess) {
+        cudaGetLastError();
+        return MPM_ERR_CUDA;
+    }
     unsigned err = 0;
     if (cudaMemcpyAsync(&err, sc.err, sizeof(unsigned), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess) {
