@@ -246,8 +246,8 @@ void L_bin(mpm_ctx *ctx, cudaStream_t st) {
     ++ctx->launches;
     ctx->bins_pending = true;
 }
-void L_between(mpm_ctx *ctx, int upd, int act, cudaStream_t st) {
-    launch_between(ctx->D, upd, act, ctx->grid_small, st);
+void L_between(mpm_ctx *ctx, int upd, int act, cudaStream_t st, bool dependent) {
+    launch_between(ctx->D, upd, act, ctx->grid_small, dependent, st);
     ++ctx->launches;
     ctx->bins_pending = false;
 }
@@ -298,15 +298,26 @@ static void middle_substep(mpm_ctx *ctx, int par, cudaStream_t st) {
 // substep on the 300k scene (61.4 with every substep ordered).
 constexpr int REORDER = 16;
 
+// Up to this many particles the two kernels of a direct-binning substep are
+// dependent launches (mpm_launch.h).  A substep then is at most about one wave
+// of CTAs (608 of 128 particles) and its launch latency counts: 100 substeps of
+// 2k, 8k, 20k, 40k and 70k particles take 8.4, 4.4, 4.5, 3.3 and 1.4% less.  A
+// larger state loses (1.9% at 120k, 11% at 300k, 22% at 2M): the persistent CTAs
+// of the substep take their places while those of k_between still hold theirs,
+// and land unevenly on the SMs.
+constexpr int DEPENDENT_MAX = 65536;
+
 // one steady-state substep s of a run with direct binning: between-substep
 // work for its buffer (grid update, work items of the last binning,
 // activation of the other buffer), then the fused G2P + P2G binning into the
 // other buffer (keep: the state it reaches is copied, so its v and C are
 // written)
-static void middle_direct(mpm_ctx *ctx, int s, cudaStream_t st, bool keep) {
+static void middle_direct(mpm_ctx *ctx, int s, cudaStream_t st, bool keep, bool follows) {
     const int par = s & 1;
-    L_between(ctx, par, par ^ 1, st);
-    L_substep(ctx, 1, par, par ^ 1, st, true, par, (keep ? SUB_KEEP : 0) | (s % REORDER ? SUB_OWN : 0));
+    const bool dep = ctx->D.n <= DEPENDENT_MAX && !ctx->trace_on;   // (a trace puts events between the launches)
+    L_between(ctx, par, par ^ 1, st, dep && follows);
+    L_substep(ctx, 1, par, par ^ 1, st, true, par,
+              (keep ? SUB_KEEP : 0) | (s % REORDER ? SUB_OWN : 0) | (dep ? SUB_DEPENDENT : 0));
 }
 
 // CUDA graph of `len` steady-state substeps: 2 (parity 0 then 1), or with
@@ -337,7 +348,7 @@ static cudaGraphExec_t steady_graph(mpm_ctx *ctx, cudaStream_t st, bool direct, 
     cudaStream_t cst = ctx->cap_stream;
     if (cudaStreamBeginCapture(cst, cudaStreamCaptureModeThreadLocal) != cudaSuccess) { cudaGetLastError(); return nullptr; }
     for (int s = 0; s < len; ++s) {
-        if (direct) middle_direct(ctx, s + 1, cst, false);
+        if (direct) middle_direct(ctx, s + 1, cst, false, s > 0);
         else middle_substep(ctx, s & 1, cst);
     }
     if (cudaStreamEndCapture(cst, &g) != cudaSuccess || !g) { cudaGetLastError(); ctx->launches = l0; return nullptr; }
@@ -398,13 +409,17 @@ mpm_status run_substeps(mpm_ctx *ctx, int n_sub, cudaStream_t st, float4 *tape, 
             ctx->launches += 2 * len;   // between + fused substep each
             return 1;
         };
+        bool follows = false;   // the last operation on the stream is a substep kernel
         for (int s = 1; s < middle;) {
             int len = 0;
             if (s % REORDER == 1 && (ctx->ran_direct || middle > 2 * REORDER)) len = replay(s, REORDER) * REORDER;
             if (!len && (s & 1) && (s + 1) % REORDER) len = replay(s, 2) * 2;
             if (len < 0) return fail(ctx, MPM_ERR_CUDA, "graph launch failed");
-            if (!len) {
-                middle_direct(ctx, s, st, due(s + 1));
+            if (len) {
+                follows = false;
+            } else {
+                middle_direct(ctx, s, st, due(s + 1), follows);
+                follows = !due(s + 1);
                 len = 1;
             }
             s += len;

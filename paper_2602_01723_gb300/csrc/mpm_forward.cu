@@ -18,6 +18,7 @@
 
 #include "mpm_dev.cuh"
 #include "mpm_internal.h"
+#include "mpm_launch.h"
 #include "mpm_math.cuh"
 
 namespace mpm {
@@ -456,6 +457,8 @@ __global__ void k_prepare(Dev D, int upd_par, int act_par, int do_sort, int keep
 // resets the ones the next substep's binning starts from.
 // ---------------------------------------------------------------------------
 __global__ void k_between(Dev D, int upd, int act) {
+    let_next_start();
+    wait_for_previous();
     const unsigned tid = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
     const unsigned nocc = D.ctr[CTR_D_OCC + upd];
     const unsigned novf = min(D.ctr[CTR_D_OVF + upd], D.ovf_cap);
@@ -753,6 +756,13 @@ __global__ void __launch_bounds__(TPB, 512 / TPB) k_substep(Dev D, int gpar, int
     constexpr bool SCATTER = MODE != MODE_G2P;
     constexpr bool PERM = SCATTER && SCAT == 1 && !OWN;        // packets taken by (rank, bank)
     constexpr bool ORDERED = GATHER && PERM;                   // particles are binned in that order
+    // the clear of the scatter tile needs nothing of the launch before (dependent
+    // launches: k_substep and k_between of a run with direct binning)
+    if (DB) let_next_start();
+    if (SCATTER && SCAT != 2)
+        for (int t = threadIdx.x; t < 4 * ST3P; t += TPB) S.t.i[t] = 0;
+    if (PERM && threadIdx.x < 32) S.ccount[threadIdx.x] = 0;
+    if (DB) wait_for_previous();
     if (DB && blockIdx.x == 0 && threadIdx.x == 0) {
         // counters this kernel does not read and the next launch starts from:
         // the activation count of the gather buffer (activated again next)
@@ -782,9 +792,6 @@ __global__ void __launch_bounds__(TPB, 512 / TPB) k_substep(Dev D, int gpar, int
         S.cd[0] = cd0;
         if (c + gridDim.x < n_chunks) S.cd[1] = cd1;
     }
-    if (SCATTER && SCAT != 2)
-        for (int t = tid; t < 4 * ST3P; t += T) S.t.i[t] = 0;
-    if (PERM && tid < 32) S.ccount[tid] = 0;
     __syncthreads();
     stage_level2<TPB, GATHER, SCATTER>(D, S, S.cd[0], gpar, spar, ep_g, ep_s);
     cp_async_commit();
@@ -1389,11 +1396,12 @@ void launch_prepare(const Dev &D, int upd_par, int act_par, int do_sort, int kee
 }
 template <int MODE, int SCAT, int TPB, bool XM, bool DB = false, bool OWN = false>
 static void launch_sub(const Dev &D, int gpar, int spar, int grid, int keep, cudaStream_t st) {
-    k_substep<MODE, SCAT, TPB, XM, DB, OWN><<<grid, TPB, substep_smem<TPB, OWN>(), st>>>(D, gpar, spar, keep);
+    launch_kernel(DB && (keep & SUB_DEPENDENT), k_substep<MODE, SCAT, TPB, XM, DB, OWN>, grid, TPB,
+                  substep_smem<TPB, OWN>(), st, D, gpar, spar, keep & SUB_KEEP);
 }
 template <int TPB>
 static void launch_tpb(const Dev &D, int mode, int gpar, int spar, int grid, bool direct, int flags, cudaStream_t st) {
-    const int keep = flags & SUB_KEEP;
+    const int keep = flags & (SUB_KEEP | SUB_DEPENDENT);   // (only SUB_KEEP reaches the kernel)
     const bool own = (flags & SUB_OWN) != 0;
     if (direct && mode == MODE_FUSED) {   // direct binning: scatter strategies 1 and 2
         if (D.xm) {
@@ -1432,8 +1440,8 @@ void launch_substep(const Dev &D, int mode, int gpar, int spar, int grid, bool d
     if (D.chunk <= 64) launch_tpb<64>(D, mode, gpar, spar, grid, direct, flags, st);
     else launch_tpb<128>(D, mode, gpar, spar, grid, direct, flags, st);
 }
-void launch_between(const Dev &D, int upd, int act, int grid, cudaStream_t st) {
-    k_between<<<grid, 256, 0, st>>>(D, upd, act);
+void launch_between(const Dev &D, int upd, int act, int grid, bool dependent, cudaStream_t st) {
+    launch_kernel(dependent, k_between, grid, 256, 0, st, D, upd, act);
 }
 void launch_export(const Dev &D, float *x, float *v, float *C, float *F, cudaStream_t st) {
     float hi, lo;

@@ -51,12 +51,13 @@ void launch_prepare(const Dev &D, int upd_par, int act_par, int do_sort, int kee
 // flags: SUB_KEEP writes v and C to the records (fused mode; G2P always does)
 // and bins the new state (G2P; the fused mode always does), SUB_OWN
 // (fixed-point scatter) scatters in list order (see k_substep)
-enum { SUB_KEEP = 1, SUB_OWN = 2 };
+// SUB_DEPENDENT (direct binning) makes it a dependent launch (mpm_launch.h)
+enum { SUB_KEEP = 1, SUB_OWN = 2, SUB_DEPENDENT = 4 };
 // direct: the fused mode bins straight into the scatter buffer's lists
 void launch_substep(const Dev &D, int mode, int gpar, int spar, int grid, bool direct, int flags, cudaStream_t st);
 // between two direct-binning substeps: grid update of upd, work items of its
 // binning, activation of act (see k_between)
-void launch_between(const Dev &D, int upd, int act, int grid, cudaStream_t st);
+void launch_between(const Dev &D, int upd, int act, int grid, bool dependent, cudaStream_t st);
 void launch_export(const Dev &D, float *x, float *v, float *C, float *F, cudaStream_t st);
 void launch_grid_dense(const Dev &D, int par, int which, float *m, float *mv, cudaStream_t st);
 int substep_occupancy(int mode, int scatter, int chunk, bool xm);
@@ -192,7 +193,7 @@ void L_prepare(mpm_ctx *ctx, int upd_par, int act_par, int do_sort, cudaStream_t
 // (G2P, or the fused mode with a sort and SUB_KEEP)
 void L_substep(mpm_ctx *ctx, int mode, int gpar, int spar, cudaStream_t st, bool direct = false, int in_par = -1,
                int flags = SUB_KEEP, float4 *rec_out = nullptr);
-void L_between(mpm_ctx *ctx, int upd, int act, cudaStream_t st);
+void L_between(mpm_ctx *ctx, int upd, int act, cudaStream_t st, bool dependent = false);
 void L_bin(mpm_ctx *ctx, cudaStream_t st);
 void launch_bgdo_accum(const Dev &D, const float4 *key, int first, float inv_k, float delta_target, float w,
                        float *G, float *g_tau, float *delta, cudaStream_t st);

@@ -22,6 +22,7 @@
 
 #include "../../include/mpm.h"
 #include "mpm_dev.cuh"
+#include "mpm_launch.h"
 #include "mpm_math.cuh"
 #include "mpm_ptr.h"
 
@@ -71,19 +72,16 @@ __device__ __forceinline__ bool locate(const Params &P, const float *x, int b[3]
 }
 
 // The substep is four dependent launches of a few microseconds: at 8k particles
-// on 32^3 their latency counts, not the work.  Each but the first is a
-// programmatic dependent launch: it starts when every CTA of the one before has
-// started, loads its inputs and does what needs nothing of that one, and waits
-// for its end before it touches the grid or the error word.  The clear, launched
-// the ordinary way, starts after all earlier work of the stream, so the inputs are
-// there; each kernel waits in every thread, so the end of one implies that of all
-// before it, and outputs that alias inputs are written after all have read them.
+// on 32^3 their latency counts, not the work.  Each but the first is a dependent
+// launch (mpm_launch.h): it loads its inputs and does what needs nothing of the
+// one before, and waits for that before it touches the grid or the error word.
+// The clear, launched the ordinary way, starts after all earlier work of the
+// stream, so the inputs are there; outputs that alias inputs are written after
+// all have read them.
 // CTAs of 64 particles: 8k particles then use 128 SMs, with 256 they used 32.
 // A call at 8k particles: 52.3 -> 43.0 us (44.3 with CTAs of 256), of which the
 // host's checks and launches and the read of the error word are some 25.
 constexpr int NA_T = 64;
-__device__ __forceinline__ void let_next_start() { cudaTriggerProgrammaticLaunchCompletion(); }
-__device__ __forceinline__ void wait_for_previous() { cudaGridDependencySynchronize(); }
 
 __global__ void k_na_clear(float4 *grid, unsigned *err, int nodes) {
     let_next_start();
@@ -253,21 +251,6 @@ __global__ void __launch_bounds__(NA_T) k_na_g2p(Params P, const float4 *grid, u
     for (int t = 0; t < 9; ++t) { C_out[9 * p + t] = Cn[t]; F_out[9 * p + t] = G[t]; }
 }
 
-// a launch that may start before the previous one in the stream has ended
-template <typename... Params_, typename... Args>
-cudaError_t launch_dependent(void (*kernel)(Params_...), int grid, int block, cudaStream_t st, Args... args) {
-    cudaLaunchAttribute attr = {};
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3((unsigned)block);
-    cfg.stream = st;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, Params_(args)...);
-}
-
 }  // namespace
 
 extern "C" MPM_API mpm_status mpm_substep_noalloc(const int32_t grid_res[3], float dx, float dt, const float gravity[3],
@@ -346,9 +329,9 @@ extern "C" MPM_API mpm_status mpm_substep_noalloc(const int32_t grid_res[3], flo
     const int ggrid = (nn + 255) / 256 < 4096 ? (nn + 255) / 256 : 4096;
     k_na_clear<<<ggrid, 256, 0, st>>>(sc.grid, sc.err, nn);
     if (cudaGetLastError() != cudaSuccess ||
-        launch_dependent(k_na_p2g, pgrid, NA_T, st, P, sc.grid, sc.err, x, v, C, F, vol, material_id) != cudaSuccess ||
-        launch_dependent(k_na_update, ggrid, 256, st, P, sc.grid, nn) != cudaSuccess ||
-        launch_dependent(k_na_g2p, pgrid, NA_T, st, P, sc.grid, sc.err, x, F, material_id, x_out, v_out, C_out, F_out) !=
+        launch_kernel(true, k_na_p2g, pgrid, NA_T, 0, st, P, sc.grid, sc.err, x, v, C, F, vol, material_id) != cudaSuccess ||
+        launch_kernel(true, k_na_update, ggrid, 256, 0, st, P, sc.grid, nn) != cudaSuccess ||
+        launch_kernel(true, k_na_g2p, pgrid, NA_T, 0, st, P, sc.grid, sc.err, x, F, material_id, x_out, v_out, C_out, F_out) !=
             cudaSuccess) {
         cudaGetLastError();
         return MPM_ERR_CUDA;
