@@ -22,6 +22,7 @@
 #include <string>
 
 #include "mpm_internal.h"
+#include "mpm_launch.h"
 #include "mpm_math.cuh"
 
 namespace mpm {
@@ -492,8 +493,10 @@ __device__ __forceinline__ void adj_stage3(const Dev &D, AdjG2PSmem &S, int4 ch,
 // per-particle bounds) and flush it with one vector reduction per touched
 // node.
 template <int MS>
-__global__ void __launch_bounds__(ADJ_THREADS, 3) k_adj_g2p(Dev D, const float4 *__restrict__ ain, float4 *aout,
+__global__ void __launch_bounds__(ADJ_THREADS, 3) k_adj_g2p(Dev D, const float4 *ain, float4 *aout,
                                                          float4 *gpar, float4 *gbar) {
+    let_next_start();
+    wait_for_previous();
     __shared__ AdjG2PSmem S;
     int4 cd0, cd1;
     first_descriptors(D, cd0, cd1);
@@ -799,6 +802,8 @@ __global__ void __launch_bounds__(ADJ_THREADS, 3) k_adj_g2p(Dev D, const float4 
 // reverse of the grid update, per active node: ubar = mask * vbar,
 // Pbar = ubar / m, mbar = -(ubar . P) / m^2; also clears the momentum pool
 __global__ void k_adj_grid(Dev D, float4 *gbar) {
+    let_next_start();
+    wait_for_previous();
     const unsigned total = min(D.ctr[CTR_N_ACTIVE + 0], D.max_active) * BLK_NODES;
     for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
         const float4 a = D.gmv[0][i];
@@ -870,6 +875,8 @@ __device__ __forceinline__ void adj_p2g_stage3(const Dev &D, AdjP2GSmem &S, int4
 // three CTAs per SM (168 registers, a few bytes of spill) measured faster than two at 216
 template <int EL>
 __global__ void __launch_bounds__(ADJ_THREADS, 3) k_adj_p2g(Dev D, float4 *aout, float4 *gpar, const float4 *gbar) {
+    let_next_start();
+    wait_for_previous();
     __shared__ AdjP2GSmem S;
     int4 cd0, cd1;
     first_descriptors(D, cd0, cd1);
@@ -1092,6 +1099,8 @@ __global__ void k_inject_tab(int n, float4 *adj, const int *frame_first, const i
 // substep s0 + j + 1
 __global__ void k_adj_between(int n, float4 *adj, const int *frame_first, const int *frame_next, const SegParams *sp,
                               int j, const unsigned *prev_ctr, unsigned max_active, float4 *gbar) {
+    let_next_start();
+    wait_for_previous();
     const unsigned tid = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
     if (prev_ctr) {
         const unsigned total = min(prev_ctr[CTR_N_ACTIVE], max_active) * BLK_NODES;
@@ -1167,6 +1176,8 @@ struct TapeSlot {
 // kernels then do nothing; the host re-runs the reverse pass with larger
 // slots.
 __global__ void k_tape_save(Dev D, int par, TapeSlot T, unsigned gcap, unsigned *over, int strict) {
+    let_next_start();
+    wait_for_previous();
     const size_t tid = blockIdx.x * (size_t)blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
     const size_t n = (size_t)D.n;
     const unsigned n_all = min(D.ctr[CTR_N_ACTIVE + par], D.max_active);
@@ -1227,19 +1238,21 @@ int adjoint_occupancy(int pl, int el) {
 }
 
 // the reverse G2P / P2G pair of the context's model set
-static void launch_adj_g2p(const mpm_ctx *ctx, const Dev &D, const float4 *ain, float4 *aout, cudaStream_t st) {
+static void launch_adj_g2p(const mpm_ctx *ctx, const Dev &D, const float4 *ain, float4 *aout, bool dependent,
+                           cudaStream_t st) {
     const AdjointStore &A = ctx->adj;
-    const int grid = ctx->grid_adj;
-    if (ctx->adj_pl == ADJ_ELASTIC) k_adj_g2p<ADJ_ELASTIC><<<grid, ADJ_THREADS, 0, st>>>(D, ain, aout, A.gpar, A.gbar);
-    else if (ctx->adj_pl == ADJ_PLASTIC) k_adj_g2p<ADJ_PLASTIC><<<grid, ADJ_THREADS, 0, st>>>(D, ain, aout, A.gpar, A.gbar);
-    else k_adj_g2p<ADJ_ALL><<<grid, ADJ_THREADS, 0, st>>>(D, ain, aout, A.gpar, A.gbar);
+    auto kernel = ctx->adj_pl == ADJ_ELASTIC ? k_adj_g2p<ADJ_ELASTIC>
+                                             : (ctx->adj_pl == ADJ_PLASTIC ? k_adj_g2p<ADJ_PLASTIC> : k_adj_g2p<ADJ_ALL>);
+    launch_kernel(dependent, kernel, ctx->grid_adj, ADJ_THREADS, 0, st, D, ain, aout, A.gpar, A.gbar);
 }
-static void launch_adj_p2g(const mpm_ctx *ctx, const Dev &D, float4 *aout, cudaStream_t st) {
+static void launch_adj_grid(const mpm_ctx *ctx, const Dev &D, bool dependent, cudaStream_t st) {
+    launch_kernel(dependent, k_adj_grid, ctx->grid_small, 256, 0, st, D, ctx->adj.gbar);
+}
+static void launch_adj_p2g(const mpm_ctx *ctx, const Dev &D, float4 *aout, bool dependent, cudaStream_t st) {
     const AdjointStore &A = ctx->adj;
-    const int grid = ctx->grid_adj;
-    if (ctx->adj_el == ADJ_FCR) k_adj_p2g<ADJ_FCR><<<grid, ADJ_THREADS, 0, st>>>(D, aout, A.gpar, A.gbar);
-    else if (ctx->adj_el == ADJ_FCR_NH) k_adj_p2g<ADJ_FCR_NH><<<grid, ADJ_THREADS, 0, st>>>(D, aout, A.gpar, A.gbar);
-    else k_adj_p2g<ADJ_ALL><<<grid, ADJ_THREADS, 0, st>>>(D, aout, A.gpar, A.gbar);
+    auto kernel = ctx->adj_el == ADJ_FCR ? k_adj_p2g<ADJ_FCR>
+                                         : (ctx->adj_el == ADJ_FCR_NH ? k_adj_p2g<ADJ_FCR_NH> : k_adj_p2g<ADJ_ALL>);
+    launch_kernel(dependent, kernel, ctx->grid_adj, ADJ_THREADS, 0, st, D, aout, A.gpar, A.gbar);
 }
 
 void free_adjoint(AdjointStore &a) {
@@ -1367,9 +1380,9 @@ static void adjoint_substep(mpm_ctx *ctx, float4 *state, float4 *ain, float4 *ao
     L_prepare(ctx, -1, 0, 1, st);
     L_substep(ctx, 0, 0, 0, st);                       // P2G of the recorded state
     L_prepare(ctx, 0, -1, 0, st, 1);                   // v = mask(mv/m + dt g), keeping (mv, m)
-    launch_adj_g2p(ctx, D, ain, aout, st);
-    k_adj_grid<<<ctx->grid_small, 256, 0, st>>>(D, A.gbar);
-    launch_adj_p2g(ctx, D, aout, st);
+    launch_adj_g2p(ctx, D, ain, aout, false, st);
+    launch_adj_grid(ctx, D, false, st);
+    launch_adj_p2g(ctx, D, aout, false, st);
     k_adj_clear<<<ctx->grid_small, 256, 0, st>>>(D, A.gbar);
     ctx->launches += 4;
     D.rec = saved;
@@ -1494,19 +1507,23 @@ static void tape_segment(mpm_ctx *ctx, int len, int bank, cudaStream_t st) {
     AdjointStore &A = ctx->adj;
     float4 *const first = ctx->D.rec;
     L_plan(ctx, 3, st);               // epochs for buffer 0 (P2G below) and 1 (first fused substep)
-    L_prepare(ctx, -1, 0, 1, st);
-    L_substep(ctx, 0, 0, 0, st);
+    // small states: dependent launches (a trace puts events between the substeps)
+    const bool dep = ctx->D.n <= DEPENDENT_MAX && !ctx->trace_on;
+    const int dep_flag = dep ? SUB_DEPENDENT : 0;
+    L_prepare(ctx, -1, 0, 1, st, 0, dep);
+    L_substep(ctx, 0, 0, 0, st, false, -1, SUB_KEEP | dep_flag);
     for (int s = 0; s < len; ++s) {
         const int par = s & 1;
         const bool more = s + 1 < len;
-        L_prepare(ctx, par, more ? par ^ 1 : -1, s > 0, st, 1);
-        k_tape_save<<<ctx->grid_small, 256, 0, st>>>(ctx->D, par, tape_slot(ctx, bank, s), A.gt_pool, gt_over(ctx),
-                                                     A.strict ? 1 : 0);
+        L_prepare(ctx, par, more ? par ^ 1 : -1, s > 0, st, 1, dep);
+        launch_kernel(dep, k_tape_save, ctx->grid_small, 256, 0, st, ctx->D, par, tape_slot(ctx, bank, s), A.gt_pool,
+                      gt_over(ctx), A.strict ? 1 : 0);
         ++ctx->launches;
         if (more) {
             float4 *const next = tape_slot(ctx, bank, s + 1).rec;
-            L_substep(ctx, 1, par, par ^ 1, st, false, -1, SUB_KEEP | (s % TAPE_REORDER ? SUB_OWN : 0), next);
-            L_plan(ctx, 1 << par, st);
+            L_substep(ctx, 1, par, par ^ 1, st, false, -1, SUB_KEEP | (s % TAPE_REORDER ? SUB_OWN : 0) | dep_flag,
+                      next);
+            L_plan(ctx, 1 << par, st, dep);
             ctx->D.rec = next;
         }
     }
@@ -1533,11 +1550,11 @@ static Dev slot_dev(mpm_ctx *ctx, const TapeSlot &T) {
 // (the grid adjoint it leaves is cleared by the next k_adj_between, or by
 // the segment's final clear)
 static void adjoint_taped(mpm_ctx *ctx, const TapeSlot &T, float4 *ain, float4 *aout, cudaStream_t st) {
-    AdjointStore &A = ctx->adj;
     const Dev Dj = slot_dev(ctx, T);
-    launch_adj_g2p(ctx, Dj, ain, aout, st);
-    k_adj_grid<<<ctx->grid_small, 256, 0, st>>>(Dj, A.gbar);
-    launch_adj_p2g(ctx, Dj, aout, st);
+    const bool dep = ctx->D.n <= DEPENDENT_MAX;
+    launch_adj_g2p(ctx, Dj, ain, aout, dep, st);
+    launch_adj_grid(ctx, Dj, dep, st);
+    launch_adj_p2g(ctx, Dj, aout, dep, st);
     ctx->launches += 3;
 }
 
@@ -1550,8 +1567,8 @@ static void reverse_segment(mpm_ctx *ctx, int len, int bank, int cur, int pg, cu
     const int n = ctx->D.n;
     for (int j = len - 1; j >= 0; --j) {
         const unsigned *prev = j + 1 < len ? tape_slot(ctx, bank, j + 1).ctr : nullptr;
-        k_adj_between<<<pg, 256, 0, st>>>(n, A.adj[cur], A.frame_first, A.frame_next, (const SegParams *)A.seg, j,
-                                          prev, ctx->D.max_active, A.gbar);
+        launch_kernel(n <= DEPENDENT_MAX && prev, k_adj_between, pg, 256, 0, st, n, A.adj[cur], A.frame_first,
+                      A.frame_next, (const SegParams *)A.seg, j, prev, ctx->D.max_active, A.gbar);
         ++ctx->launches;
         adjoint_taped(ctx, tape_slot(ctx, bank, j), A.adj[cur], A.adj[cur ^ 1], st);
         cur ^= 1;

@@ -232,13 +232,14 @@ mpm_status mpm::ensure_chunks(mpm_ctx *ctx) {
 // ===========================================================================
 namespace mpm {
 
-void L_plan(mpm_ctx *ctx, int bump_mask, cudaStream_t st) {
-    launch_plan(ctx->D, bump_mask, st);
+void L_plan(mpm_ctx *ctx, int bump_mask, cudaStream_t st, bool dependent) {
+    launch_plan(ctx->D, bump_mask, dependent, st);
     ++ctx->launches;
     ctx->bins_pending = false;
 }
-void L_prepare(mpm_ctx *ctx, int upd_par, int act_par, int do_sort, cudaStream_t st, int keep_momentum) {
-    launch_prepare(ctx->D, upd_par, act_par, do_sort, keep_momentum, ctx->grid_small, st);
+void L_prepare(mpm_ctx *ctx, int upd_par, int act_par, int do_sort, cudaStream_t st, int keep_momentum,
+               bool dependent) {
+    launch_prepare(ctx->D, upd_par, act_par, do_sort, keep_momentum, ctx->grid_small, dependent, st);
     ++ctx->launches;
 }
 void L_bin(mpm_ctx *ctx, cudaStream_t st) {
@@ -297,15 +298,6 @@ static void middle_substep(mpm_ctx *ctx, int par, cudaStream_t st) {
 // order decays slowly: 4, 16 and 1000 measured 57.5, 57.0 and 57.9 us per
 // substep on the 300k scene (61.4 with every substep ordered).
 constexpr int REORDER = 16;
-
-// Up to this many particles the two kernels of a direct-binning substep are
-// dependent launches (mpm_launch.h).  A substep then is at most about one wave
-// of CTAs (608 of 128 particles) and its launch latency counts: 100 substeps of
-// 2k, 8k, 20k, 40k and 70k particles take 8.4, 4.4, 4.5, 3.3 and 1.4% less.  A
-// larger state loses (1.9% at 120k, 11% at 300k, 22% at 2M): the persistent CTAs
-// of the substep take their places while those of k_between still hold theirs,
-// and land unevenly on the SMs.
-constexpr int DEPENDENT_MAX = 65536;
 
 // one steady-state substep s of a run with direct binning: between-substep
 // work for its buffer (grid update, work items of the last binning,

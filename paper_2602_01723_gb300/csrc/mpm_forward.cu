@@ -303,6 +303,8 @@ __device__ __forceinline__ void block_scan2(unsigned a, unsigned b, unsigned &ea
 }
 
 __global__ void __launch_bounds__(1024) k_plan(Dev D, int bump_mask) {
+    let_next_start();
+    wait_for_previous();
     __shared__ unsigned sh[66];
     const unsigned n = D.ctr[CTR_N_OCC];
     const unsigned CH = (unsigned)D.chunk;
@@ -406,6 +408,8 @@ __device__ __forceinline__ void apply_walls(const Dev &D, int I, int J, int K, f
 }
 
 __global__ void k_prepare(Dev D, int upd_par, int act_par, int do_sort, int keep_momentum) {
+    let_next_start();
+    wait_for_previous();
     const unsigned tid = blockIdx.x * blockDim.x + threadIdx.x, stride = gridDim.x * blockDim.x;
     // each warp takes one kind of item (a grid node, an activation neighbour,
     // a particle to sort), ranges rounded up to whole warps: no thread chains
@@ -756,13 +760,12 @@ __global__ void __launch_bounds__(TPB, 512 / TPB) k_substep(Dev D, int gpar, int
     constexpr bool SCATTER = MODE != MODE_G2P;
     constexpr bool PERM = SCATTER && SCAT == 1 && !OWN;        // packets taken by (rank, bank)
     constexpr bool ORDERED = GATHER && PERM;                   // particles are binned in that order
-    // the clear of the scatter tile needs nothing of the launch before (dependent
-    // launches: k_substep and k_between of a run with direct binning)
-    if (DB) let_next_start();
+    // the clear of the scatter tile needs nothing of the launch before
+    let_next_start();
     if (SCATTER && SCAT != 2)
         for (int t = threadIdx.x; t < 4 * ST3P; t += TPB) S.t.i[t] = 0;
     if (PERM && threadIdx.x < 32) S.ccount[threadIdx.x] = 0;
-    if (DB) wait_for_previous();
+    wait_for_previous();
     if (DB && blockIdx.x == 0 && threadIdx.x == 0) {
         // counters this kernel does not read and the next launch starts from:
         // the activation count of the gather buffer (activated again next)
@@ -1390,13 +1393,16 @@ void launch_load(const Dev &D, const LoadArgs &a, cudaStream_t st) {
     k_load<<<grid_for(D.n, IO_T), IO_T, 0, st>>>(D, hi, lo, a.x, a.v, a.C, a.F, a.vol, a.mat, a.inst, a.params, a.table);
 }
 void launch_bin(const Dev &D, cudaStream_t st) { k_bin<<<grid_for(D.n, 256), 256, 0, st>>>(D); }
-void launch_plan(const Dev &D, int bump_mask, cudaStream_t st) { k_plan<<<1, 1024, 0, st>>>(D, bump_mask); }
-void launch_prepare(const Dev &D, int upd_par, int act_par, int do_sort, int keep_momentum, int grid, cudaStream_t st) {
-    k_prepare<<<grid, 256, 0, st>>>(D, upd_par, act_par, do_sort, keep_momentum);
+void launch_plan(const Dev &D, int bump_mask, bool dependent, cudaStream_t st) {
+    launch_kernel(dependent, k_plan, 1, 1024, 0, st, D, bump_mask);
+}
+void launch_prepare(const Dev &D, int upd_par, int act_par, int do_sort, int keep_momentum, int grid, bool dependent,
+                    cudaStream_t st) {
+    launch_kernel(dependent, k_prepare, grid, 256, 0, st, D, upd_par, act_par, do_sort, keep_momentum);
 }
 template <int MODE, int SCAT, int TPB, bool XM, bool DB = false, bool OWN = false>
 static void launch_sub(const Dev &D, int gpar, int spar, int grid, int keep, cudaStream_t st) {
-    launch_kernel(DB && (keep & SUB_DEPENDENT), k_substep<MODE, SCAT, TPB, XM, DB, OWN>, grid, TPB,
+    launch_kernel((keep & SUB_DEPENDENT) != 0, k_substep<MODE, SCAT, TPB, XM, DB, OWN>, grid, TPB,
                   substep_smem<TPB, OWN>(), st, D, gpar, spar, keep & SUB_KEEP);
 }
 template <int TPB>

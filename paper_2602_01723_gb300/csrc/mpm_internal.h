@@ -46,12 +46,22 @@ inline int grid_for(long long n, int threads, int cap = 152 * 16) {
 
 void launch_load(const Dev &D, const LoadArgs &a, cudaStream_t st);   // bins the particles too
 void launch_bin(const Dev &D, cudaStream_t st);
-void launch_plan(const Dev &D, int bump_mask, cudaStream_t st);
-void launch_prepare(const Dev &D, int upd_par, int act_par, int do_sort, int keep_momentum, int grid, cudaStream_t st);
+void launch_plan(const Dev &D, int bump_mask, bool dependent, cudaStream_t st);
+void launch_prepare(const Dev &D, int upd_par, int act_par, int do_sort, int keep_momentum, int grid, bool dependent,
+                    cudaStream_t st);
+// Up to this many particles the kernels of a direct-binning substep, and those of
+// a taped segment and of its reverse, are dependent launches (mpm_launch.h).  A
+// substep then is at most about one wave of CTAs (608 of 128 particles) and its
+// launch latency counts: 100 substeps of 2k, 8k, 20k, 40k and 70k particles take
+// 8.4, 4.4, 4.5, 3.3 and 1.4% less, a gradient pass of 512 and of 50k particles
+// 2.4 and 1.8%.  A larger state loses (1.9% at 120k, 11% at 300k, 22% at 2M): the
+// persistent CTAs of the substep take their places while those of k_between still
+// hold theirs, and land unevenly on the SMs.
+constexpr int DEPENDENT_MAX = 65536;
 // flags: SUB_KEEP writes v and C to the records (fused mode; G2P always does)
 // and bins the new state (G2P; the fused mode always does), SUB_OWN
 // (fixed-point scatter) scatters in list order (see k_substep)
-// SUB_DEPENDENT (direct binning) makes it a dependent launch (mpm_launch.h)
+// SUB_DEPENDENT makes it a dependent launch (mpm_launch.h)
 enum { SUB_KEEP = 1, SUB_OWN = 2, SUB_DEPENDENT = 4 };
 // direct: the fused mode bins straight into the scatter buffer's lists
 void launch_substep(const Dev &D, int mode, int gpar, int spar, int grid, bool direct, int flags, cudaStream_t st);
@@ -184,9 +194,10 @@ namespace mpm {
 // kernel launches through these wrappers are counted (and the substep kernel
 // timed when tracing is on)
 // plan of the current grouping; opens fresh epochs for the buffers in bump_mask
-void L_plan(mpm_ctx *ctx, int bump_mask, cudaStream_t st);
+void L_plan(mpm_ctx *ctx, int bump_mask, cudaStream_t st, bool dependent = false);
 // grid update of upd_par, activation of act_par, sorted index (see k_prepare)
-void L_prepare(mpm_ctx *ctx, int upd_par, int act_par, int do_sort, cudaStream_t st, int keep_momentum = 0);
+void L_prepare(mpm_ctx *ctx, int upd_par, int act_par, int do_sort, cudaStream_t st, int keep_momentum = 0,
+               bool dependent = false);
 // direct: bin straight into the scatter buffer's lists (fused mode); in_par
 // >= 0: read the work items of the direct binning into buffer in_par;
 // rec_out: write the new records there and leave the state's as they are
