@@ -207,8 +207,8 @@ MPM_API mpm_status mpm_reduce_by_material(mpm_ctx *ctx, const float *per_particl
 
 /* Sets the substep kernel's tuning: scatter strategy (0, 1, 2 as in
  * mpm_options), particles per work chunk (a multiple of 16 in [16, 128]) and
- * whether steady-state substeps replay a CUDA graph (two substeps per graph
- * launch; tracing disables the graph). */
+ * whether steady-state substeps replay a CUDA graph (two or sixteen substeps
+ * per graph launch; tracing disables the graph). */
 MPM_API mpm_status mpm_set_tuning(mpm_ctx *ctx, int32_t scatter, int32_t chunk, int32_t use_graph);
 
 /* Autotuner: times n_substeps >= 2 substeps from the current state for each
