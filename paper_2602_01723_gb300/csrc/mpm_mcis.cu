@@ -367,7 +367,7 @@ constexpr int FIRST_RINGS = 2;     // reach of the first pass, unless the first 
 constexpr int DIRECT_RINGS = 4;    // this close already
 constexpr int SAMPLES = 8;         // surface points each lane tries for a first bound
 struct WarpScratch {
-    unsigned cell[1024];           // occupied cells still to be read: mask word << 5 | bit
+    unsigned cell[1024];           // occupied cells still to be read: mask word of the object << 5 | bit
     float4 pt[32];                 // points (x y z, index) that every candidate meets
     float two[TURN / 2][8];        // candidates 2 u, 2 u + 1: x x y y z z, bounds
     unsigned char order[32];       // candidates by (cell, octant of the cell)
@@ -469,6 +469,11 @@ __device__ __forceinline__ void search(Near3 &m, bool active, float qx, float qy
                                        float cut2, const Grid &g, const Cells &C, WarpScratch &W) {
     const int lane = threadIdx.x & 31;
     const float hf = 1.f / g.inv_h;
+    // words are counted from the object's first: one object's mask has at most
+    // 2^23 (512 cells per axis would be 4.5M), so that a cell's number fits 32
+    // bits, while all objects together may have more than 2^27
+    const long long words0 = mask_row(g, p.k, 0, 0);
+    const unsigned *const mask = C.mask + words0, *const before = C.before + words0;
     seed = fminf(seed, cut2);
     auto bound = [&]() {   // squared distance beyond which no candidate needs a point, with the margin of FP32 box distances
         seed = fminf(seed, m.d1);
@@ -503,15 +508,15 @@ __device__ __forceinline__ void search(Near3 &m, bool active, float qx, float qy
             const int ix = (int)(((float)c + 0.5f) * iw);   // c / wy: c < 2^10, never near an integer
             const int x = X0 + ix, y = Y0 + c - ix * wy;
             unsigned bits = 0;             // occupied cells z0 .. z1 of the row that belong to this pass
-            unsigned at = 0;               // of z0's cell: mask word << 5 | bit
+            unsigned at = 0;               // of z0's cell: mask word of the object << 5 | bit
             // a row at the cube's face also holds what lies beyond it and is always looked up
             if (c < rows && x >= 0 && y >= 0 && x < g.G && y < g.G &&
                 (x == 0 || y == 0 || x == g.G - 1 || y == g.G - 1 ||
                  gap2(p.a[0], p.b[0], (float)x * hf, (float)(x + 1) * hf) +
                          gap2(p.a[1], p.b[1], (float)y * hf, (float)(y + 1) * hf) <= worst)) {
-                const long long row = mask_row(g, p.k, x, y) + (z0 >> 5);
-                at = (unsigned)row << 5 | (z0 & 31);
-                bits = __funnelshift_r(C.mask[row], C.mask[row + 1], z0 & 31) & all;
+                const unsigned row = (unsigned)((x * g.G + y) * g.zwords + (z0 >> 5));
+                at = row << 5 | (z0 & 31);
+                bits = __funnelshift_r(mask[row], mask[row + 1], z0 & 31) & all;
                 if (x >= p.c0[0] - done && x <= p.c1[0] + done && y >= p.c0[1] - done && y <= p.c1[1] + done) bits &= ~old;
             }
             if (__any_sync(0xffffffffu, bits != 0)) {
@@ -536,7 +541,7 @@ __device__ __forceinline__ void search(Near3 &m, bool active, float qx, float qy
                 float dist = INFINITY;
                 if (lane < take) {
                     const unsigned e = W.cell[listed + lane];
-                    const unsigned c = C.before[e >> 5] + __popc(C.mask[e >> 5] & ((1u << (e & 31)) - 1u));
+                    const unsigned c = before[e >> 5] + __popc(mask[e >> 5] & ((1u << (e & 31)) - 1u));
                     lo = C.lo[c];
                     hi = C.hi[c];
                     dist = gap2(p.a[0], p.b[0], lo.x, hi.x) + gap2(p.a[1], p.b[1], lo.y, hi.y) +
