@@ -15,8 +15,12 @@
 //     time, and search rings of cells in order of distance until the best
 //     distance is below the ring's lower bound.  Beyond
 //     d_cut = sigma sqrt(2 ln(1/eps)) the weight is eps whatever the
-//     distance, so the search radius is d_cut.  Distances are screened in
-//     FP32 and confirmed in FP64, so the minimum is the exact FP64 one;
+//     distance, so the search radius is d_cut.  Distances are compared in
+//     FP32; the points that FP32 cannot tell apart from the nearest are settled
+//     in FP64 at the end, so the minimum is the exact FP64 one.  A second kernel
+//     takes the candidates with nothing within d_cut, whose distance is that to
+//     the nearest point in the coarse cells around them, and those with many
+//     points at the same distance;
 //   * weights are summed as integers round(w 2^40), which makes the
 //     cumulative sums independent of the summation order, and each draw
 //     binary-searches its object's cumulative sums for floor(u W_k).
@@ -246,73 +250,8 @@ __device__ __forceinline__ double dist2(float qx, float qy, float qz, float4 c) 
     return fx * fx + fy * fy + fz * fz;
 }
 
-// Squared distance to the nearest surface point in the coarse cells up to RINGS
-// away, every decision in FP64; one thread.  For a candidate with nothing
-// within d_cut (the coarse cells then say how far it looked), or whose three
-// nearest points agree to FP32 rounding (repeated points).
-__device__ __noinline__ double nn_exact(float qx, float qy, float qz, int k, const Grid &g, const Cells &C) {
-    const int Gc = g.G / g.sub;
-    const float inv_hc = g.inv_h / (float)g.sub;
-    const double h = 1.0 / (double)inv_hc;
-    const float hf = 1.f / inv_hc;
-    const int cx = cell_of(qx, inv_hc, Gc), cy = cell_of(qy, inv_hc, Gc), cz = cell_of(qz, inv_hc, Gc);
-    double best = INFINITY;
-    float screen = INFINITY;   // best * (1 + 1e-6), rounded up to FP32
-    for (int r = 0; r <= RINGS; ++r) {
-        // cells of ring r lie at least (r - 1) h away: stop once the best is closer
-        const double lb = (double)(r - 1) * h;
-        if (r > 1 && best <= lb * lb) break;
-        // pruning threshold in FP32: the FP32 box distance of a cell within d_cut is
-        // within 1.3e-7 of the exact one (cell edges and differences rounded), so this
-        // margin never skips a cell that could hold a closer point
-        const float prune = (float)best * 1.00001f + 2e-7f;
-        for (int ix = -r; ix <= r; ++ix) {
-            const int x = cx + ix;
-            if (x < 0 || x >= Gc) continue;
-            for (int iy = -r; iy <= r; ++iy) {
-                const int y = cy + iy;
-                if (y < 0 || y >= Gc) continue;
-                // ring r only: the whole row on its x or y faces, else its two z ends
-                const bool face = ix == -r || ix == r || iy == -r || iy == r;
-                const int zstep = (face || r == 0) ? 1 : 2 * r;
-                for (int iz = -r; iz <= r; iz += zstep) {
-                    const int z = cz + iz;
-                    if (z < 0 || z >= Gc) continue;
-                    // a cell wholly farther than the best point holds nothing closer
-                    // (cells are clamped at the cube's faces, so only interior cells are skipped)
-                    if (x > 0 && y > 0 && z > 0 && x < Gc - 1 && y < Gc - 1 && z < Gc - 1 &&
-                        box_d2f(qx, x, hf) + box_d2f(qy, y, hf) + box_d2f(qz, z, hf) > prune)
-                        continue;
-                    for (int a = 0; a < g.sub * g.sub * g.sub; ++a) {   // its cells
-                        const int fz = z * g.sub + a % g.sub, fy = y * g.sub + a / g.sub % g.sub, fx = x * g.sub + a / (g.sub * g.sub);
-                        const long long w = mask_row(g, k, fx, fy) + (fz >> 5);
-                        const unsigned word = C.mask[w], bit = 1u << (fz & 31);
-                        if (!(word & bit)) continue;
-                        const unsigned c = C.before[w] + __popc(word & (bit - 1u));
-                        const float4 lo = C.lo[c], hi = C.hi[c];
-                        if (range_d2f(qx, lo.x, hi.x) + range_d2f(qy, lo.y, hi.y) + range_d2f(qz, lo.z, hi.z) > prune) continue;
-                        const unsigned s0 = __float_as_uint(lo.w), s1 = s0 + __float_as_uint(hi.w);
-                        for (unsigned s = s0; s < s1; ++s) {
-                            const float4 t = C.point[s];
-                            const float ex = qx - t.x, ey = qy - t.y, ez = qz - t.z;
-                            const float d2f = ex * ex + ey * ey + ez * ez;
-                            // the FP32 value is within 1e-6 relative of the exact one, so a
-                            // point closer than best passes this FP32 screen
-                            if (d2f <= screen) {
-                                const double d2 = dist2(qx, qy, qz, t);
-                                if (d2 < best) {
-                                    best = d2;
-                                    screen = __double2float_ru(best * (1.0 + 1e-6));
-                                }
-                            }
-                        }
-                    }
-                }
-            }
-        }
-    }
-    return best;
-}
+// device counters: the scans' ticket, then candidates and items left to k_mc_open, its next item
+enum { OPEN_COUNT = 1, OPEN_ITEMS, OPEN_NEXT, MC_COUNTERS };
 
 // the three smallest FP32 squared distances seen, with the points of the two
 // smallest; a NaN is never kept
@@ -403,6 +342,23 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
 __device__ __forceinline__ float2 range_pair(float2 q, float lo, float nhi) {
     const float2 over = add2(q, make_float2(nhi, nhi));
     return make_float2(fmaxf(0.f, fmaxf(lo - q.x, over.x)), fmaxf(0.f, fmaxf(lo - q.y, over.y)));
+}
+
+// Appends every lane's cells to the warp's list, each as `at` plus its bit's
+// number; the list's new length.  The whole warp.
+__device__ __forceinline__ int list_cells(unsigned *cell, int listed, unsigned bits, unsigned at) {
+    const int lane = threadIdx.x & 31;
+    unsigned incl = __popc(bits);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned u = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += u;
+    }
+    __syncwarp();
+    for (int to = listed + (int)incl - __popc(bits); bits; bits &= bits - 1) cell[to++] = at + (unsigned)(__ffs(bits) - 1);
+    listed += (int)__shfl_sync(0xffffffffu, incl, 31);
+    __syncwarp();
+    return listed;
 }
 
 // Distances from the lanes' candidates to the points of the cells of the lanes
@@ -520,17 +476,7 @@ __device__ __forceinline__ void search(Near3 &m, bool active, float qx, float qy
                 if (x >= p.c0[0] - done && x <= p.c1[0] + done && y >= p.c0[1] - done && y <= p.c1[1] + done) bits &= ~old;
             }
             if (__any_sync(0xffffffffu, bits != 0)) {
-                unsigned incl = __popc(bits);
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const unsigned u = __shfl_up_sync(0xffffffffu, incl, o);
-                    if (lane >= o) incl += u;
-                }
-                __syncwarp();
-                for (int to = listed + (int)incl - __popc(bits); bits; bits &= bits - 1)
-                    W.cell[to++] = at + (unsigned)(__ffs(bits) - 1);
-                listed += (int)__shfl_sync(0xffffffffu, incl, 31);
-                __syncwarp();
+                listed = list_cells(W.cell, listed, bits, at);
             }
             // 32 cells at a time, what is left over after the last row
             const bool last = c0 + 32 >= rows;
@@ -614,10 +560,10 @@ __device__ __forceinline__ void search(Near3 &m, bool active, float qx, float qy
 // (divergent), 32 candidates of one lane each 1.3 ms (a few deep groups, whose
 // points are nearly equidistant, ran twice as long as all others).
 constexpr int GROUP = 2;
-__global__ void __launch_bounds__(32 * NN_WARPS) k_mc_nn(int n_obj, const int64_t *soff, const int64_t *coff,
+__global__ void __launch_bounds__(32 * NN_WARPS, 7) k_mc_nn(int n_obj, const int64_t *soff, const int64_t *coff,
                                                          const float *cand, const unsigned *order, Grid g, Cells C,
                                                          int per, int reach, float cells_sorted, float cut2,
-                                                         double *d2) {
+                                                         uint2 *open, uint2 *items, unsigned *ctr, double *d2) {
     __shared__ WarpScratch scratch[NN_WARPS];
     WarpScratch &W = scratch[threadIdx.x >> 5];
     const int64_t n = coff[n_obj];
@@ -663,6 +609,7 @@ __global__ void __launch_bounds__(32 * NN_WARPS) k_mc_nn(int n_obj, const int64_
     const bool mine = (lane >> 2) < per && k >= 0;
     const int cx = cell_of(qx, g.inv_h, g.G), cy = cell_of(qy, g.inv_h, g.G), cz = cell_of(qz, g.inv_h, g.G);
     double best = INFINITY;
+    bool opened = false;   // the lane's candidate is left to k_mc_open
     unsigned todo = __ballot_sync(0xffffffffu, mine);   // four bits per candidate
     while (todo) {
         const int lead = __ffs(todo) - 1;
@@ -734,7 +681,8 @@ __global__ void __launch_bounds__(32 * NN_WARPS) k_mc_nn(int n_obj, const int64_
         }
         const float limit = fmaf(d1, 3e-6f, d1) + 1e-36f;
         double e = INFINITY;
-        bool again = active && !(d1 < INFINITY && d1 <= cut2 * 0.99997f);   // nothing within d_cut (cut2 carries a margin of 1e-5)
+        const bool none = !(d1 < INFINITY && d1 <= cut2 * 0.99997f);   // nothing within d_cut (cut2 carries a margin of 1e-5)
+        bool again = active && none;
         if (active && !again) {
             if (m.d1 <= limit) e = dist2(px, py, pz, C.point[m.i1]);
             if (m.d2 <= limit) e = fmin(e, dist2(px, py, pz, C.point[m.i2]));
@@ -742,15 +690,322 @@ __global__ void __launch_bounds__(32 * NN_WARPS) k_mc_nn(int n_obj, const int64_
         }
         const unsigned crowd = __ballot_sync(0xffffffffu, again);
         for (int o = 1; o < (together ? 4 : 32); o <<= 1) e = fmin(e, __shfl_xor_sync(0xffffffffu, e, o));
-        if (together) {
-            if (active && (lane & 3) == 0 && ((crowd >> lane) & 0xfu)) e = nn_exact(px, py, pz, p.k, g, C);
-            if (active) best = e;
-        } else if (lane == lead) {
-            best = crowd ? nn_exact(px, py, pz, p.k, g, C) : e;
+        // left to k_mc_open: those with nothing within d_cut, together, and the
+        // others still open, one by one
+        if (crowd) {
+            const unsigned heads = together ? 0x11111111u : 1u << lead;   // the candidates' first lanes
+            const unsigned far = __ballot_sync(0xffffffffu, again && none) & heads;
+            const unsigned quad = crowd | crowd >> 1 | crowd >> 2 | crowd >> 3;
+            const unsigned left = together ? quad & heads : heads, alone = left & ~far;
+            unsigned o0 = 0, i0 = 0;
+            if (lane == 0) {
+                o0 = atomicAdd(&ctr[OPEN_COUNT], (unsigned)__popc(left));
+                i0 = atomicAdd(&ctr[OPEN_ITEMS], (unsigned)__popc(alone) + (far ? 1u : 0u));
+            }
+            o0 = __shfl_sync(0xffffffffu, o0, 0);
+            i0 = __shfl_sync(0xffffffffu, i0, 0);
+            if ((far >> lane) & 1u) {
+                const unsigned r = __popc(far & lanes_before());
+                open[o0 + r] = make_uint2((unsigned)j, __float_as_uint(INFINITY));
+                if (r == 0) items[i0] = make_uint2(o0, (unsigned)__popc(far));
+            }
+            o0 += __popc(far);
+            i0 += far ? 1 : 0;
+            if ((alone >> lane) & 1u) {
+                const unsigned r = __popc(alone & lanes_before());
+                open[o0 + r] = make_uint2((unsigned)j, __float_as_uint(limit));
+                items[i0 + r] = make_uint2(o0 + r, 1u | 1u << 4);
+            }
+            if ((left >> lane) & 1u) opened = true;
         }
+        if (together ? active : lane == lead) best = e;
         __syncwarp();
     }
-    if (mine && (lane & 3) == 0) d2[j] = best;
+    if (mine && (lane & 3) == 0 && !opened) d2[j] = best;
+}
+
+// the smallest of the lanes' values
+__device__ __forceinline__ double warp_min(double x) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x = fmin(x, __shfl_xor_sync(0xffffffffu, x, o));
+    return x;
+}
+
+// the cells a .. b of a grid, up to 31 along z
+struct Window {
+    int a[3], b[3];
+    __device__ __forceinline__ int rows() const { return (b[0] - a[0] + 1) * (b[1] - a[1] + 1); }
+    __device__ __forceinline__ void row(int r, int &x, int &y) const {
+        const int wy = b[1] - a[1] + 1;
+        x = a[0] + r / wy;
+        y = a[1] + r % wy;
+    }
+};
+// occupied cells of row (x, y) of a window; word: of its first cell
+__device__ __forceinline__ unsigned row_bits(const Window &w, const Grid &g, const Cells &C, int k, int x, int y, long long &word) {
+    word = mask_row(g, k, x, y) + (w.a[2] >> 5);
+    return __funnelshift_r(C.mask[word], C.mask[word + 1], w.a[2] & 31) & (0xffffffffu >> (31 - (w.b[2] - w.a[2])));
+}
+// box of the occupied cell z cells behind a window's first in a row
+__device__ __forceinline__ void cell_box(const Window &w, const Cells &C, long long word, int z, float4 &lo, float4 &hi) {
+    const int at = (w.a[2] & 31) + z;
+    word += at >> 5;
+    const unsigned c = C.before[word] + __popc(C.mask[word] & ((1u << (at & 31)) - 1u));
+    lo = C.lo[c];
+    hi = C.hi[c];
+}
+// the cells of the coarse cells up to RINGS away from a candidate's
+__device__ __forceinline__ Window coarse_window(float qx, float qy, float qz, const Grid &g) {
+    const int Gc = g.G / g.sub;
+    const float inv_hc = g.inv_h / (float)g.sub;
+    const int c[3] = {cell_of(qx, inv_hc, Gc), cell_of(qy, inv_hc, Gc), cell_of(qz, inv_hc, Gc)};
+    Window w;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        w.a[d] = max(c[d] - RINGS, 0) * g.sub;
+        w.b[d] = min(c[d] + RINGS, Gc - 1) * g.sub + g.sub - 1;
+    }
+    return w;
+}
+
+// Squared distance of one candidate to its nearest surface point, decided in
+// FP64; the whole warp.  For a candidate whose three nearest points agree to FP32
+// rounding (repeated points).  limit: an FP32 squared distance that the nearest
+// point does not exceed.  Each lane looks up a row of the cells within the limit
+// and holds the box of one occupied cell at a time against the best distance; the
+// points of a cell are shared out over the lanes.
+__device__ __forceinline__ double nn_exact(float qx, float qy, float qz, float limit, int k, const Grid &g, const Cells &C) {
+    const int lane = threadIdx.x & 31;
+    const float hf = 1.f / g.inv_h;
+    // a point beyond the cube is in the cube's outermost cells, as q -+ reach then is
+    const float reach = sqrtf(limit) * 1.00001f + 1e-6f, q[3] = {qx, qy, qz};
+    Window w = coarse_window(qx, qy, qz, g);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        w.a[d] = max(w.a[d], cell_of(q[d] - reach, g.inv_h, g.G));
+        w.b[d] = min(w.b[d], cell_of(q[d] + reach, g.inv_h, g.G));
+    }
+    double best = INFINITY;
+    float screen = limit;   // best * (1 + 1e-6), rounded up to FP32
+    // pruning threshold in FP32: the FP32 distance of a box within d_cut is within
+    // 1.3e-7 of the exact one (cell edges and differences rounded), so this margin
+    // never skips a cell that could hold a closer point
+    float prune = limit * 1.00001f + 2e-7f;
+    const int rows = w.rows();
+    for (int r0 = 0; r0 < rows; r0 += 32) {
+        unsigned bits = 0;
+        long long word = 0;
+        int x, y;
+        w.row(r0 + lane, x, y);
+        // (a row at the cube's face also holds what lies beyond it)
+        if (r0 + lane < rows && (x == 0 || y == 0 || x == g.G - 1 || y == g.G - 1 ||
+                                 box_d2f(qx, x, hf) + box_d2f(qy, y, hf) <= prune))
+            bits = row_bits(w, g, C, k, x, y, word);
+        while (__any_sync(0xffffffffu, bits != 0)) {
+            bool near = false;
+            unsigned s0 = 0, n = 0;
+            if (bits) {
+                float4 lo, hi;
+                cell_box(w, C, word, __ffs(bits) - 1, lo, hi);
+                bits &= bits - 1;
+                near = range_d2f(qx, lo.x, hi.x) + range_d2f(qy, lo.y, hi.y) + range_d2f(qz, lo.z, hi.z) <= prune;
+                s0 = __float_as_uint(lo.w);
+                n = __float_as_uint(hi.w);
+            }
+            for (unsigned keep = __ballot_sync(0xffffffffu, near); keep; keep &= keep - 1) {
+                const int l = __ffs(keep) - 1;
+                const unsigned p0 = __shfl_sync(0xffffffffu, s0, l), m = __shfl_sync(0xffffffffu, n, l);
+                for (unsigned i = lane; i < m; i += 32) {
+                    const float4 t = C.point[p0 + i];
+                    const float ex = qx - t.x, ey = qy - t.y, ez = qz - t.z;
+                    // the FP32 value is within 1e-6 relative of the exact one, so a
+                    // point closer than best passes this FP32 screen
+                    if (ex * ex + ey * ey + ez * ez <= screen) best = fmin(best, dist2(qx, qy, qz, t));
+                }
+            }
+            best = warp_min(best);
+            if (best < INFINITY) {
+                screen = fminf(screen, __double2float_ru(best * (1.0 + 1e-6)));
+                prune = fminf(prune, (float)best * 1.00001f + 2e-7f);
+            }
+        }
+    }
+    return best;
+}
+
+constexpr int OPEN_WARPS = 4;      // warps per CTA
+struct FarScratch {
+    unsigned cell[1024];           // occupied cells still to be read: row of the window << 5 | z
+    struct {
+        float q[3], bound;
+        int a[3], b[3];
+    } far[TURN];
+};
+// Squared distances of the lanes' candidates (one per four lanes, those of `mine`)
+// to the nearest surface points in their coarse windows, decided in FP64
+// (INFINITY: none); the whole warp.  For candidates with nothing within d_cut:
+// their windows then say how far they looked.  The candidates walk the occupied
+// cells of all their windows together, 32 at a time, a cell per lane: once for a
+// limit per candidate, the farthest corner of the box that is nearest by it, then
+// for the points of the boxes within it.
+__device__ __forceinline__ double nn_far(bool mine, float qx, float qy, float qz, int k, const Grid &g, const Cells &C,
+                                         FarScratch &W) {
+    const int lane = threadIdx.x & 31, own = lane >> 2;
+    const float q[3] = {qx, qy, qz};
+    Window o = coarse_window(qx, qy, qz, g);
+    __syncwarp();
+    if ((lane & 3) == 0) {
+        auto &f = W.far[own];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            f.q[d] = q[d];
+            f.a[d] = o.a[d];
+            f.b[d] = o.b[d];
+        }
+        f.bound = INFINITY;
+    }
+    __syncwarp();
+    float limit[TURN];
+#pragma unroll
+    for (int u = 0; u < TURN; ++u) limit[u] = INFINITY;
+    bool held = false, odd = false;   // an occupied cell; one with a point that is not finite, whose box says nothing
+    double best = INFINITY;
+    for (int walk = 0; walk < 2; ++walk) {
+        float screen = W.far[own].bound;
+        if (walk) {
+            // the cells within the limits; a point beyond the cube is in the cube's
+            // outermost cells, as q -+ reach then is
+            mine = mine && (odd || screen < INFINITY);
+            const float reach = sqrtf(screen) * 1.00001f + 1e-6f;
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                o.a[d] = max(o.a[d], cell_of(q[d] - reach, g.inv_h, g.G));
+                o.b[d] = min(o.b[d], cell_of(q[d] + reach, g.inv_h, g.G));
+            }
+        }
+        const unsigned them = __ballot_sync(0xffffffffu, mine);
+        if (!them) break;
+        Window w;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            w.a[d] = __reduce_min_sync(0xffffffffu, mine ? o.a[d] : g.G);
+            w.b[d] = __reduce_max_sync(0xffffffffu, mine ? o.b[d] : 0);
+        }
+        const int rows = w.rows();
+        int listed = 0;   // cells in the list: row << 5 | z
+        for (int r0 = 0; r0 < rows; r0 += 32) {
+            unsigned bits = 0;
+            if (r0 + lane < rows) {
+                int x, y;
+                long long word;
+                w.row(r0 + lane, x, y);
+                bits = row_bits(w, g, C, k, x, y, word);
+            }
+            if (__any_sync(0xffffffffu, bits != 0)) listed = list_cells(W.cell, listed, bits, (unsigned)(r0 + lane) << 5);
+            // 32 cells at a time, what is left over after the last row
+            const bool last = r0 + 32 >= rows;
+            while (listed >= 32 || (last && listed > 0)) {
+                const int take = min(listed, 32);
+                listed -= take;
+                unsigned wanted = 0;   // candidates that need this lane's cell
+                unsigned s0 = 0, n = 0;
+                if (lane < take) {
+                    const unsigned e = W.cell[listed + lane];
+                    const int z = e & 31, zz = w.a[2] + z;
+                    int x, y;
+                    w.row(e >> 5, x, y);
+                    float4 lo, hi;
+                    cell_box(w, C, mask_row(g, k, x, y) + (w.a[2] >> 5), z, lo, hi);
+                    s0 = __float_as_uint(lo.w);
+                    n = __float_as_uint(hi.w);
+                    held = true;
+                    odd |= !isfinite((hi.x - lo.x) + (hi.y - lo.y) + (hi.z - lo.z));
+#pragma unroll
+                    for (int u = 0; u < TURN; ++u) {
+                        const auto &f = W.far[u];
+                        if (!((them >> (4 * u)) & 1u)) continue;
+                        if (x < f.a[0] || x > f.b[0] || y < f.a[1] || y > f.b[1] || zz < f.a[2] || zz > f.b[2]) continue;
+                        if (walk == 0) {
+                            const float fx = fmaxf(hi.x - f.q[0], f.q[0] - lo.x), fy = fmaxf(hi.y - f.q[1], f.q[1] - lo.y),
+                                        fz = fmaxf(hi.z - f.q[2], f.q[2] - lo.z);
+                            limit[u] = fminf(limit[u], fx * fx + fy * fy + fz * fz);
+                        } else if (range_d2f(f.q[0], lo.x, hi.x) + range_d2f(f.q[1], lo.y, hi.y) +
+                                       range_d2f(f.q[2], lo.z, hi.z) <= f.bound * 1.00001f + 2e-7f) {
+                            wanted |= 1u << u;
+                        }
+                    }
+                }
+                __syncwarp();
+                if (walk == 0) continue;
+                for (unsigned keep = __ballot_sync(0xffffffffu, wanted != 0); keep; keep &= keep - 1) {
+                    const int l = __ffs(keep) - 1;
+                    const unsigned p0 = __shfl_sync(0xffffffffu, s0, l), m = __shfl_sync(0xffffffffu, n, l);
+                    if ((__shfl_sync(0xffffffffu, wanted, l) >> own) & 1u)
+                        for (unsigned i = lane & 3; i < m; i += 4) {
+                            const float4 t = C.point[p0 + i];
+                            const float ex = qx - t.x, ey = qy - t.y, ez = qz - t.z;
+                            // (the FP32 value is within 1e-6 relative of the exact one)
+                            if (ex * ex + ey * ey + ez * ez <= screen) {
+                                const double d2 = dist2(qx, qy, qz, t);
+                                if (d2 < best) {
+                                    best = d2;
+                                    screen = fminf(screen, __double2float_ru(best * (1.0 + 1e-6)));
+                                }
+                            }
+                        }
+                }
+            }
+        }
+        if (walk == 0) {
+            if (!__any_sync(0xffffffffu, held)) return INFINITY;   // deep inside an object
+            odd = __any_sync(0xffffffffu, odd);
+            __syncwarp();
+#pragma unroll
+            for (int u = 0; u < TURN; ++u) {
+                // with the margin of the FP32 distances of the points
+                const float t = odd ? INFINITY : warp_min(limit[u]) * 1.00001f + 1e-36f;
+                if (lane == 0) W.far[u].bound = t;
+            }
+            __syncwarp();
+        }
+    }
+    best = fmin(best, __shfl_xor_sync(0xffffffffu, best, 1));
+    return fmin(best, __shfl_xor_sync(0xffffffffu, best, 2));
+}
+
+// The candidates that k_mc_nn leaves open: an item is a group of up to TURN of them
+// with nothing within d_cut, or one whose nearest points FP32 cannot tell apart
+// (y >> 4); open: candidate and limit.  A warp takes the next item when it is done
+// with one, since some walk a few cells and some hundreds.
+//
+// In a kernel of its own so that the search keeps its registers (with both in one
+// the search spilled 146 bytes, and a ball of radius 0.3 took 2.2 ms).  Fills of
+// 250k candidates and 36,000 surface points, by one thread per candidate without
+// occupied cells, with one lane per open candidate walking its window after the
+// search, and so: a ball of radius 0.3, 27% of the candidates beyond d_cut, 1.5,
+// 72.8 and 1.2 ms; a ball of radius 0.15, 3%, 2.3, 8.9 and 1.3 ms; every surface
+// point three times, 5.3, 6.8 and 1.6 ms.
+__global__ void __launch_bounds__(32 * OPEN_WARPS) k_mc_open(int n_obj, const int64_t *coff, const float *cand, Grid g, Cells C,
+                                                             const uint2 *open, const uint2 *items, unsigned *ctr,
+                                                             double *d2) {
+    __shared__ FarScratch scratch[OPEN_WARPS];
+    const int lane = threadIdx.x & 31;
+    for (;;) {
+        unsigned i = 0;
+        if (lane == 0) i = atomicAdd(&ctr[OPEN_NEXT], 1u);
+        i = __shfl_sync(0xffffffffu, i, 0);
+        if (i >= ctr[OPEN_ITEMS]) return;
+        const uint2 item = items[i];
+        const unsigned n = item.y & 15u;
+        const bool one = (item.y >> 4) != 0, mine = (unsigned)(lane >> 2) < n;
+        const uint2 o = open[item.x + (mine ? lane >> 2 : 0)];
+        const int64_t j = o.x;
+        const float qx = cand[3 * j], qy = cand[3 * j + 1], qz = cand[3 * j + 2];
+        const int k = find_range(coff, n_obj, j);
+        const double x = one ? nn_exact(qx, qy, qz, __uint_as_float(o.y), k, g, C)
+                             : nn_far(mine, qx, qy, qz, k, g, C, scratch[threadIdx.x >> 5]);
+        if (mine && (lane & 3) == 0) d2[j] = x;
+    }
 }
 
 // step 2: distance, weight and integer weight of the squared distance, in place
@@ -864,8 +1119,8 @@ extern "C" MPM_API mpm_status mpm_mcis(int32_t n_obj, const int64_t *surf_off, c
     const size_t o_surf = off; off += al(ns * 12);
     const size_t o_cand = off; off += al(nc * 12);
     const size_t o_u = off; off += al(nd * 8);
-    // cleared together: the scans' ticket, mask, points per cell, boxes, candidates per cell
-    const size_t o_ticket = off; off += al(4);
+    // cleared together: counters, mask, points per cell, boxes, candidates per cell
+    const size_t o_ticket = off; off += al(MC_COUNTERS * 4);
     const size_t o_mask = off; off += al(words * 4);
     const size_t o_cnt = off; off += al(ns * 4);
     const size_t o_box = off; off += al(ns * 24);
@@ -882,6 +1137,8 @@ extern "C" MPM_API mpm_status mpm_mcis(int32_t n_obj, const int64_t *surf_off, c
     const size_t o_ccell = off; off += al(nc * 4);
     const size_t o_crank = off; off += al(nc * 4);
     const size_t o_order = off; off += al(nc * 4);
+    const size_t o_open = off; off += al(nc * 8);
+    const size_t o_items = off; off += al(nc * 8);
     const size_t o_sorted = off; off += al(ns * 16);
     const size_t o_wq = off; off += al(nc * 8);
     const size_t o_cum = off; off += al(nc * 8);
@@ -950,7 +1207,10 @@ extern "C" MPM_API mpm_status mpm_mcis(int32_t n_obj, const int64_t *surf_off, c
             const int per = (int)std::min<long long>(TURN, std::max<long long>(1, nc / (152 * 24)));
             const long long ctas = (nc + per * NN_WARPS - 1) / (per * NN_WARPS);
             k_mc_nn<<<(unsigned)ctas, 32 * NN_WARPS, 0, st>>>(n_obj, dsoff, dcoff, dcand, order, g, cells, per,
-                                                              std::max(1, g.sub / 2), (float)Gs, cut2, (double *)wq);
+                                                              std::max(1, g.sub / 2), (float)Gs, cut2,
+                                                              (uint2 *)P(o_open), (uint2 *)P(o_items), ticket, (double *)wq);
+            k_mc_open<<<(unsigned)std::min<long long>(152 * 5, (nc + OPEN_WARPS - 1) / OPEN_WARPS), 32 * OPEN_WARPS, 0, st>>>(
+                n_obj, dcoff, dcand, g, cells, (const uint2 *)P(o_open), (const uint2 *)P(o_items), ticket, (double *)wq);
             k_mc_weight<<<blocks_for(nc, 256), 256, 0, st>>>(nc, sigma, eps, dd, dw, wq);
             MC_CK(cudaGetLastError());
             k_mc_scan_i64_block<<<(unsigned)nb, 1024, 0, st>>>(wq, cum, nc, tot);
