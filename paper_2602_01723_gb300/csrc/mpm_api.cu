@@ -864,11 +864,12 @@ MPM_API mpm_status mpm_autotune(mpm_ctx *ctx, int32_t n_substeps, int32_t out[3]
     // 64-thread CTAs at twice the CTAs per SM, larger ones 128-thread CTAs)
     const int scats[2] = {1, 2}, chunks[4] = {32, 64, 96, 128};
     mpm_status s = MPM_OK;
+    ctx->ran_direct = true;   // from the first trial on, the warm-up captures every graph that the timed pass replays
     for (int a = 0; a < 2 && !s; ++a)
         for (int b = 0; b < 4 && !s; ++b) {
             if ((s = mpm_set_tuning(ctx, scats[a], chunks[b], graph0))) break;
             float ms = 0.f;
-            for (int rep = 0; rep < 2 && !s; ++rep) {   // first pass warms up (and captures the graph)
+            for (int rep = 0; rep < 2 && !s; ++rep) {   // first pass warms up (and captures the graphs)
                 CK(cudaMemcpyAsync(D.rec, snap, bytes, cudaMemcpyDeviceToDevice, st));
                 L_plan(ctx, 0, st);
                 L_bin(ctx, st);
