@@ -30,7 +30,7 @@
  *
  *  - mpm_mcis and mpm_render, which have no context, take their scratch from a
  *    memory pool of the library's that keeps up to 256 MiB per device between
- *    calls; destroying the last context gives it back.
+ *    calls; destroying the last context or mpm_release_scratch gives it back.
  *
  * Errors
  *  - Every entry point returns mpm_status; no C++ exception crosses the ABI.
@@ -333,6 +333,11 @@ MPM_API mpm_status mpm_render(int64_t n, const float *mean, const float *cov, co
                               int32_t width, int32_t height, const float bg[3], float *image, float *trans,
                               void *stream);
 MPM_API const char *mpm_render_last_error(void);
+
+/* Gives the scratch memory that mpm_mcis and mpm_render have kept on every
+ * device back (for a program that makes no context; the next such call takes
+ * it anew).  Safe at any time: memory in use stays. */
+MPM_API mpm_status mpm_release_scratch(void);
 
 /* Diagnostic: P2G of the current state into dense device arrays m
  * (n_instances * R0 * R1 * R2 floats, node (b, I, J, K) at

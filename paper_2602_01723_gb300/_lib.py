@@ -77,6 +77,7 @@ SIGNATURES = {
     "mpm_render": (ctypes.c_int, [ctypes.c_int64, _vp, _vp, _vp, _vp, _f32p, ctypes.c_float, ctypes.c_float,
                                   ctypes.c_float, ctypes.c_float, ctypes.c_int32, ctypes.c_int32, _f32p, _vp, _vp, _vp]),
     "mpm_render_last_error": (ctypes.c_char_p, []),
+    "mpm_release_scratch": (ctypes.c_int, []),
     "mpm_set_tuning": (ctypes.c_int, [_ctx_p, ctypes.c_int32, ctypes.c_int32, ctypes.c_int32]),
     "mpm_autotune": (ctypes.c_int, [_ctx_p, ctypes.c_int32, _i32p, _vp]),
     "mpm_substep_noalloc": (ctypes.c_int, [_i32p, ctypes.c_float, ctypes.c_float, _f32p, ctypes.POINTER(mpm_material),

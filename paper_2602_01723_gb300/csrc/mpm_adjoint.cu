@@ -24,6 +24,7 @@
 #include "mpm_internal.h"
 #include "mpm_launch.h"
 #include "mpm_math.cuh"
+#include "mpm_scratch.h"
 
 namespace mpm {
 
@@ -1289,7 +1290,7 @@ static mpm_status checkpoint_slot(mpm_ctx *ctx, size_t c, cudaStream_t st) {
                                                 "recorded run at least as long");
         if (A.ckpt[c]) cudaFree(A.ckpt[c]);
         A.ckpt[c] = nullptr;
-        cudaError_t e = cudaMalloc(&A.ckpt[c], bytes);
+        cudaError_t e = device_alloc((void **)&A.ckpt[c], bytes);
         if (e != cudaSuccess) {
             cudaGetLastError();
             A.ckpt[c] = nullptr;
@@ -1358,7 +1359,7 @@ template <typename T>
 static mpm_status dev_alloc(mpm_ctx *ctx, T **p, size_t count) {
     if (*p) cudaFree(*p);
     *p = nullptr;
-    cudaError_t e = cudaMalloc((void **)p, (count ? count : 1) * sizeof(T));
+    cudaError_t e = device_alloc((void **)p, (count ? count : 1) * sizeof(T));
     if (e != cudaSuccess) {
         cudaGetLastError();
         *p = nullptr;
@@ -1469,7 +1470,7 @@ static bool ensure_grid_tape(mpm_ctx *ctx, size_t states, cudaStream_t st) {
     const unsigned pool = gt_pool_for(ctx, st);
     size_t off[9];
     const size_t slot = gt_layout(ctx, pool, off), bytes = GT_HEADER + 2 * states * slot;
-    if (cudaMalloc(&A.gt, bytes) != cudaSuccess) {
+    if (device_alloc((void **)&A.gt, bytes) != cudaSuccess) {
         cudaGetLastError();
         A.gt = nullptr;
         return false;
@@ -1813,7 +1814,7 @@ extern "C" MPM_API mpm_status mpm_backward(mpm_ctx *ctx, int32_t n_frames, const
         A.frame_cap = std::max(n_frames, 1);
     }
     if (!A.seg) {
-        if (cudaMalloc(&A.seg, sizeof(SegParams)) != cudaSuccess) {
+        if (device_alloc((void **)&A.seg, sizeof(SegParams)) != cudaSuccess) {
             cudaGetLastError();
             A.seg = nullptr;
             return ctx_fail(ctx, MPM_ERR_OOM, "reverse-pass allocation failed");

@@ -52,7 +52,7 @@ template <typename T>
 mpm_status dalloc(mpm_ctx *ctx, T **p, size_t count, bool zero) {
     if (*p) { cudaFree(*p); *p = nullptr; }
     if (count == 0) count = 1;
-    cudaError_t e = cudaMalloc((void **)p, count * sizeof(T));
+    cudaError_t e = device_alloc((void **)p, count * sizeof(T));
     if (e != cudaSuccess) {
         *p = nullptr;
         cudaGetLastError();
@@ -126,7 +126,7 @@ mpm_status ensure_stage(mpm_ctx *ctx, size_t bytes) {
     if (bytes <= ctx->stage_bytes) return MPM_OK;
     dfree(ctx->stage);
     ctx->stage_bytes = 0;
-    cudaError_t e = cudaMalloc(&ctx->stage, bytes);
+    cudaError_t e = device_alloc((void **)&ctx->stage, bytes);
     if (e != cudaSuccess) { cudaGetLastError(); ctx->stage = nullptr; return fail(ctx, MPM_ERR_OOM, "staging allocation failed"); }
     ctx->stage_bytes = bytes;
     return MPM_OK;
@@ -849,7 +849,7 @@ MPM_API mpm_status mpm_autotune(mpm_ctx *ctx, int32_t n_substeps, int32_t out[3]
     float4 *snap = (float4 *)ctx->stage;
     bool own = false;
     if (bytes > ctx->stage_bytes) {
-        if (cudaMalloc(&snap, bytes) != cudaSuccess) { cudaGetLastError(); return fail(ctx, MPM_ERR_OOM, "autotune snapshot"); }
+        if (device_alloc((void **)&snap, bytes) != cudaSuccess) { cudaGetLastError(); return fail(ctx, MPM_ERR_OOM, "autotune snapshot"); }
         own = true;
     }
     CK(cudaMemcpyAsync(snap, D.rec, bytes, cudaMemcpyDeviceToDevice, st));
@@ -893,6 +893,11 @@ MPM_API mpm_status mpm_autotune(mpm_ctx *ctx, int32_t n_substeps, int32_t out[3]
     if (s2) return s2;
     if (s3) return s3;
     if (out) { out[0] = D.scatter; out[1] = D.chunk; out[2] = (int32_t)(best * 1000.f); }
+    return MPM_OK;
+}
+
+MPM_API mpm_status mpm_release_scratch(void) {
+    scratch_trim();
     return MPM_OK;
 }
 

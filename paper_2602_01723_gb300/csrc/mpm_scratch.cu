@@ -45,8 +45,10 @@ cudaError_t scratch_alloc(void **p, size_t bytes, cudaStream_t st) {
         const cudaMemPool_t pool = pool_of(device);
         if (pool) {
             const cudaError_t e = cudaMallocFromPoolAsync(p, bytes, pool, st);
-            // out of memory with the pool's own reserve: the default pool has none to offer either
-            if (e == cudaSuccess || e == cudaErrorMemoryAllocation) return e;
+            if (e == cudaSuccess) return e;
+            // out of memory: what this pool keeps in pieces too small goes back, and
+            // the default pool may hold memory that another user has freed into it
+            if (e == cudaErrorMemoryAllocation) cudaMemPoolTrimTo(pool, 0);
         }
     }
     cudaGetLastError();
@@ -57,6 +59,16 @@ void scratch_trim() {
     std::lock_guard<std::mutex> lock(g_mutex);
     for (cudaMemPool_t p : g_pool)
         if (p && cudaMemPoolTrimTo(p, 0) != cudaSuccess) cudaGetLastError();
+}
+
+cudaError_t device_alloc(void **p, size_t bytes) {
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        scratch_trim();
+        e = cudaMalloc(p, bytes);
+    }
+    return e;
 }
 
 }  // namespace mpm
