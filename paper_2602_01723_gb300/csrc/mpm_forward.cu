@@ -129,19 +129,6 @@ template <int W> __device__ __forceinline__ void stage_rows(float *dst, const fl
     }
 }
 
-// x in fixed-point units, rounded to the nearest: x cells_hi + x cells_lo, where
-// hi + lo are units per world length, as a float pair.  The product's rounding
-// error is recovered by a multiply-add, so that the sum carries about 48 bits;
-// (in FP64 the division and the conversion kept the FP64 pipe 80% busy)
-__device__ __forceinline__ int to_fixed(float x, float hi, float lo) {
-    float p = x * hi;
-    if (!isfinite(p)) return isinf(x) || !isinf(p) ? 0 : (p > 0.f ? 1073741824 : -1073741824);
-    if (fabsf(p) >= 1073741824.f) return p > 0.f ? 1073741824 : -1073741824;
-    const float e = fmaf(x, hi, -p) + x * lo;
-    const float t = rintf(p);
-    return (int)t + (int)rintf((p - t) + e);
-}
-
 // Records are put together in shared memory and written 128 bytes at a time by
 // neighbouring lanes, the caller's arrays are read the same way: bound by DRAM.
 // 2M particles: 181 us + 81 us of binning -> 136 us for both.
@@ -200,7 +187,7 @@ __global__ void __launch_bounds__(IO_T) k_load(Dev D, float units_hi, float unit
             for (int d = 0; d < 3; ++d) {
                 const float xd = in[3 * tid + d];
                 fin = fin && isfinite(xd);
-                q[d] = to_fixed(xd, units_hi, units_lo);
+                q[d] = to_fixed(xd, units_hi, units_lo, D.dx, D.q_cell);
             }
             const float *vv = in + 3 * IO_T + 3 * tid;
             r[0] = make_float4(__int_as_float(q[0]), __int_as_float(q[1]), __int_as_float(q[2]), rho * vp);
@@ -1278,23 +1265,16 @@ template <int W> __device__ __forceinline__ void unstage_rows(float *dst, const 
     if (dst)
         for (int t = threadIdx.x; t < cnt * W; t += IO_T) dst[(size_t)p0 * W + t] = src[t];
 }
-// fixed point -> world units, rounded once to FP32: the position and the unit
-// each as a float pair
-__device__ __forceinline__ float to_world(int q, float unit_hi, float unit_lo) {
-    const float h = (float)q, l = (float)(q - (int)h);
-    const float p = h * unit_hi;
-    return p + (fmaf(h, unit_hi, -p) + fmaf(h, unit_lo, l * unit_hi));
-}
 // positions alone, one word of each record: a frame of a trajectory or a splat
-__global__ void __launch_bounds__(256) k_export_x(Dev D, float unit_hi, float unit_lo, float *__restrict__ x) {
+__global__ void __launch_bounds__(256) k_export_x(Dev D, float unit, float *__restrict__ x) {
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < D.n; p += gridDim.x * blockDim.x) {
         const float4 r0 = D.rec[(size_t)p * REC_F4];
-        x[3 * (size_t)p] = to_world(rec_q(r0.x), unit_hi, unit_lo);
-        x[3 * (size_t)p + 1] = to_world(rec_q(r0.y), unit_hi, unit_lo);
-        x[3 * (size_t)p + 2] = to_world(rec_q(r0.z), unit_hi, unit_lo);
+        x[3 * (size_t)p] = to_world(rec_q(r0.x), unit);
+        x[3 * (size_t)p + 1] = to_world(rec_q(r0.y), unit);
+        x[3 * (size_t)p + 2] = to_world(rec_q(r0.z), unit);
     }
 }
-__global__ void __launch_bounds__(IO_T) k_export(Dev D, float unit_hi, float unit_lo, float *x, float *v, float *C, float *F) {
+__global__ void __launch_bounds__(IO_T) k_export(Dev D, float unit, float *x, float *v, float *C, float *F) {
     __shared__ float4 rec[IO_T * IO_F4];
     __shared__ float out[IO_T * 24];
     const int tid = threadIdx.x;
@@ -1313,9 +1293,9 @@ __global__ void __launch_bounds__(IO_T) k_export(Dev D, float unit_hi, float uni
             const float4 *r = rec + tid * IO_F4;
             if (x) {
                 const float4 r0 = r[0];
-                out[3 * tid] = to_world(rec_q(r0.x), unit_hi, unit_lo);
-                out[3 * tid + 1] = to_world(rec_q(r0.y), unit_hi, unit_lo);
-                out[3 * tid + 2] = to_world(rec_q(r0.z), unit_hi, unit_lo);
+                out[3 * tid] = to_world(rec_q(r0.x), unit);
+                out[3 * tid + 1] = to_world(rec_q(r0.y), unit);
+                out[3 * tid + 2] = to_world(rec_q(r0.z), unit);
             }
             float *o = out + 3 * IO_T + 3 * tid;
             if (v) { const float4 r1 = r[1]; o[0] = r1.x; o[1] = r1.y; o[2] = r1.z; }
@@ -1450,10 +1430,9 @@ void launch_between(const Dev &D, int upd, int act, int grid, bool dependent, cu
     launch_kernel(dependent, k_between, grid, 256, 0, st, D, upd, act);
 }
 void launch_export(const Dev &D, float *x, float *v, float *C, float *F, cudaStream_t st) {
-    float hi, lo;
-    float_pair((double)D.q_unit * (double)D.dx, hi, lo);
-    if (x && !v && !C && !F) k_export_x<<<grid_for(D.n, 256), 256, 0, st>>>(D, hi, lo, x);
-    else k_export<<<grid_for(D.n, IO_T), IO_T, 0, st>>>(D, hi, lo, x, v, C, F);
+    const float unit = D.q_unit * D.dx;   // (exact: q_unit is a power of two)
+    if (x && !v && !C && !F) k_export_x<<<grid_for(D.n, 256), 256, 0, st>>>(D, unit, x);
+    else k_export<<<grid_for(D.n, IO_T), IO_T, 0, st>>>(D, unit, x, v, C, F);
 }
 void launch_grid_dense(const Dev &D, int par, int which, float *m, float *mv, cudaStream_t st) {
     k_grid_dense<<<1024, 256, 0, st>>>(D, par, which, m, mv);
