@@ -1089,22 +1089,28 @@ extern "C" MPM_API mpm_status mpm_mcis(int32_t n_obj, const int64_t *surf_off, c
     if (g.G < 1) g.G = 1;
     if (g.G > 256) g.G = 256;
     if ((long long)g.G * g.G * g.G * n_obj >= (1ll << 31)) { g_mcis_msg = "mcis: grid too large"; return MPM_ERR_INVALID_ARG; }
-    // twice as fine where an object has the points to fill the cells (36,000
-    // points an object: 1.5 ms for 750k candidates, 2.1 ms with coarse cells,
-    // 1.7 ms four times as fine), while the mask stays within 8M words (its
-    // clearing and scan then cost some 30 us)
+    // twice as fine where an object has the points to fill the cells, while the mask
+    // stays within 8M words (its clearing and scan then cost some 30 us).  Three
+    // objects, coarse and fine: 4,000 points each and 50k candidates 324 and 367 us,
+    // 12,000 and 250k 650 and 656, 36,000 and 250k 1,189 and 1,072.  A ball of
+    // radius 0.1, 250k candidates: 12,000 points 555 and 595 us, 18,000 692 and 715,
+    // 25,000 949 and 883, 36,000 1,555 and 1,248.  (A ball of 0.2, whose points are
+    // sparser, gains from 100,000 points on.)
     const int Gc = g.G;
     auto mask_words = [&](int sub) {
         const long long G = (long long)Gc * sub;
         return n_obj * G * G * ((G + 31) / 32 + 1);
     };
-    g.sub = ns / n_obj >= 2000 && mask_words(2) <= (1ll << 23) ? 2 : 1;
+    g.sub = ns / n_obj >= 24000 && mask_words(2) <= (1ll << 23) ? 2 : 1;
     g.G = Gc * g.sub;
     g.inv_h = (float)g.G;
     g.zwords = (g.G + 31) / 32 + 1;
     const long long words = mask_words(g.sub);
     const float cut2 = (float)(cut * cut * (1.0 + 1e-5));
-    // the candidates' cells: up to twice the coarse grid's, about a warp's worth in one
+    // the candidates' cells: up to twice the coarse grid's, about a warp's worth in
+    // one.  Coarse and twice as fine, a ball with 36,000 points: 12k candidates 687
+    // and 829 us, 25k 772 and 920, 50k 985 and 877, 100k 1,140 and 1,170; 4,000
+    // points: 25k 351 and 364, 50k 348 and 317, 100k 381 and 353
     int Gs = Gc;
     if (8ll * Gc * Gc * Gc * n_obj <= (1ll << 23) && nc / n_obj >= 50000) Gs *= 2;
     const long long keys = (long long)n_obj * Gs * Gs * Gs;
