@@ -1368,8 +1368,6 @@ static mpm_status dev_alloc(mpm_ctx *ctx, T **p, size_t count) {
     return MPM_OK;
 }
 
-// consume any pending binning, then bin the current records
-
 // reverse of one substep whose input state is `state`
 static void adjoint_substep(mpm_ctx *ctx, float4 *state, float4 *ain, float4 *aout, cudaStream_t st) {
     Dev &D = ctx->D;

@@ -52,11 +52,14 @@ void launch_prepare(const Dev &D, int upd_par, int act_par, int do_sort, int kee
 // Up to this many particles the kernels of a direct-binning substep, and those of
 // a taped segment and of its reverse, are dependent launches (mpm_launch.h).  A
 // substep then is at most about one wave of CTAs (608 of 128 particles) and its
-// launch latency counts: 100 substeps of 2k, 8k, 20k, 40k and 70k particles take
-// 8.4, 4.4, 4.5, 3.3 and 1.4% less, a gradient pass of 512 and of 50k particles
-// 2.4 and 1.8%.  A larger state loses (1.9% at 120k, 11% at 300k, 22% at 2M): the
-// persistent CTAs of the substep take their places while those of k_between still
-// hold theirs, and land unevenly on the SMs.
+// launch latency counts: 100 substeps of 2k, 8k, 20k, 40k, 50k, 65k and 70k particles
+// take 8.4, 4.4, 4.5, 3.3, 2.5, 2.1 and 1.9% less.  Beyond one wave it depends on
+// the state (85k in one object 2.3% less, 77k in three objects 1.1% more) and
+// turns into a loss (100k 3.3, 120k 2.4, 300k 11, 2M 22% more): the persistent
+// CTAs of the substep take their places while those of k_between still hold
+// theirs, and land unevenly on the SMs.  A gradient pass of 512 and of 50k particles
+// on 64^3 takes 2.4 and 1.8% less, of 50k on 96^3 0.5 and of 65k 0.3% more, of 70k
+// 1.7 and of 77k 3.8% more.
 constexpr int DEPENDENT_MAX = 65536;
 // flags: SUB_KEEP writes v and C to the records (fused mode; G2P always does)
 // and bins the new state (G2P; the fused mode always does), SUB_OWN
