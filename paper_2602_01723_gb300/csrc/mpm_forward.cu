@@ -566,9 +566,9 @@ __global__ void k_between(Dev D, int upd, int act) {
 //      (OWN) scatter each thread's own particle from registers in list order,
 //      without packets, their sort and two of the five barriers, and their
 //      gather reads distinct banks as well.
-// What bounds it: the shared-memory data pipe (70% busy at 300k particles
-// before the gather tile became planes, the tile strides covered all banks and
-// the unread v and C stores went; 59% after) and, with 16 warps per SM, the
+// What bounds it: the load/store data pipe (53% busy at 300k particles, 43% with
+// shared memory, after the gather tile became planes, the tile strides covered all
+// banks and the unread v and C stores went) and, with 16 warps per SM, the
 // latency of one particle's dependent chain.  Fused launch 62.5 -> 53.4 us at
 // 300k particles on 128^3 and 356 -> 297 us at 2M on 256^3 (53 and 58% of the
 // issue slots unused; DRAM 8 and 21%).

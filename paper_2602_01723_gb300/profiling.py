@@ -112,6 +112,8 @@ WANT = [
     ("smsp__inst_executed.sum", "warp instructions"),
     ("smsp__inst_executed_op_shared_atom.sum", "shared atomic instructions"),
     ("l1tex__t_requests_pipe_lsu_mem_global_op_red.sum", "global reduction requests"),
+    ("l1tex__data_pipe_lsu_wavefronts.avg.pct_of_peak_sustained_elapsed", "load/store data pipe %"),
+    ("l1tex__data_pipe_lsu_wavefronts_mem_shared.avg.pct_of_peak_sustained_elapsed", "... of it for shared memory"),
     ("launch__registers_per_thread", "registers / thread"),
     ("launch__grid_size", "grid"),
     ("launch__block_size", "block"),
